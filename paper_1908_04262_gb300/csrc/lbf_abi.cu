@@ -90,7 +90,7 @@ struct lbf_sim {
   int *lab_fast = nullptr;
   int *lab_full = nullptr;
   bool walled = false;  // walls close every face and no fluid cell lies in a face layer
-  int *rmv = nullptr;
+  int *rmv = nullptr, *rmlist = nullptr, *rank = nullptr;
   int tile_blocks = 0;
   uint8_t *tdirty = nullptr;
   size_t ntiles_alloc = 0;
@@ -192,6 +192,8 @@ Params make_params(lbf_sim *s, long long step) {
   p.lab_fast = s->lab_fast;
   p.lab_full = s->lab_full;
   p.rmv = s->rmv;
+  p.rmlist = s->rmlist;
+  p.rank = s->rank;
   p.tile_blocks = s->tile_blocks;
   p.tdirty = s->tdirty;
   p.rlabel = s->rlabel;
@@ -363,18 +365,14 @@ void enqueue_after_sweep(lbf_sim *s, const Params &p, int par, bool waitx, const
     mark_low_priority(s, s->st3);
     cudaEventRecord(s->joinx, s->st3);
   }
-  // the labelling branch is chosen on the device after the marking (see
-  // k_label_choose): the kernels of the branch not taken return at once
-  s->ops->label_choose(p, s->st);
+  // the labelling branch is chosen on the device by the labelling check; the
+  // union-find kernels, which return at once in a patched step, run while
+  // the excess is collected
   s->ops->label_forest(p, s->st);
   cudaStreamWaitEvent(s->st, s->applied, 0);
-  // the patch first: ready with the excess collection, it goes ahead of the
-  // geometry's blocks (the relabelling of the other branch returns at once)
-  s->ops->label_fast(p, s->st);
   s->ops->label_relabel(p, s->st);
   cudaEventRecord(s->fork[1], s->st);
   s->ops->bubble_update(p, s->st);
-  s->ops->bubble_update_fast(p, s->st);
   cudaStreamWaitEvent(s->st4, s->fork[1], 0);
   cudaStreamWaitEvent(s->st4, s->join[0], 0);
   s->ops->disjoining(pn, s->st4);
@@ -419,14 +417,9 @@ void enqueue_step(lbf_sim *s, const Params &p, int par, cudaEvent_t *ev) {
   });
   const Params pn = next_geometry_params(p);
   group(G_LABEL, [&] {
-    s->ops->label_choose(p, s->st);
     s->ops->label(p, s->st);
-    s->ops->label_fast(p, s->st);
   });
-  group(G_BUBBLE, [&] {
-    s->ops->bubble_update(p, s->st);
-    s->ops->bubble_update_fast(p, s->st);
-  });
+  group(G_BUBBLE, [&] { s->ops->bubble_update(p, s->st); });
   group(G_GEOMETRY, [&] { enqueue_geometry(s, pn, s->st); });
   group(G_DISJOIN, [&] { s->ops->disjoining(pn, s->st); });
 }
@@ -717,13 +710,17 @@ int validate(const lbf_config *c) {
 namespace lbf {
 void set_last_error(const char *msg) { g_err = msg; }
 
-// the bubble table as lbf_bubble rows after a 16-byte header holding the
-// row count
+// the bubble table as lbf_bubble rows, in the order of the roots (a row is
+// the count of smaller roots), after a 16-byte header holding the row count
 __global__ void k_pack_bubbles(Table t, unsigned char *out, int rows) {
   const int nb = *t.count;
   if (blockIdx.x == 0 && threadIdx.x == 0) *reinterpret_cast<int *>(out) = nb;
   lbf_bubble *r = reinterpret_cast<lbf_bubble *>(out + 16);
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < rows && i < nb; i += gridDim.x * blockDim.x) {
+  __shared__ int sr[1024];
+  for (int i0 = blockIdx.x * blockDim.x; i0 < nb; i0 += gridDim.x * blockDim.x) {
+    const int i = i0 + (int)threadIdx.x;
+    const int row = count_below(t.root, nb, i < nb ? t.root[i] : 0, sr);
+    if (i >= nb || row >= rows) continue;
     lbf_bubble b;
     b.id = t.id[i];
     b.atm = t.atm[i];
@@ -731,12 +728,34 @@ __global__ void k_pack_bubbles(Table t, unsigned char *out, int rows) {
     b.volume = t.V[i];
     b.gas_mass = t.m[i];
     b.pressure = t.p[i];
-    r[i] = b;
+    r[row] = b;
   }
 }
-void pack_bubbles_launch(const Table &t, unsigned char *out, int rows, cudaStream_t st) {
-  const int blocks = rows > 0 ? (rows + 255) / 256 : 1;
-  k_pack_bubbles<<<blocks, 256, 0, st>>>(t, out, rows);
+void pack_bubbles_launch(const Table &t, unsigned char *out, int rows, int cap, cudaStream_t st) {
+  k_pack_bubbles<<<(cap + 255) / 256, 256, 0, st>>>(t, out, rows);
+}
+
+// the labels and the bubble table in the order of the roots: cells, then
+// rows into the table `to` (whose accumulators the caller clears again)
+__global__ void k_order_labels(const int *rank, int *label, long long N) {
+  for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < N; n += (long long)gridDim.x * blockDim.x) {
+    const int l = label[n];
+    if (l >= 0) label[n] = rank[l];
+  }
+}
+__global__ void k_order_table(Table t, const int *rank, Table to) {
+  const int nb = *t.count;
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nb; i += gridDim.x * blockDim.x) {
+    const int r = rank[i];
+    to.m[r] = t.m[i];
+    to.p[r] = t.p[i];
+    to.V[r] = t.V[i];
+    to.dm[r] = t.dm[i];
+    to.id[r] = t.id[i];
+    to.atm[r] = t.atm[i];
+    to.root[r] = t.root[i];
+    to.ng[r] = t.ng[i];
+  }
 }
 
 // checks a staged lbf_set_cells input before it replaces the state: bit 0 a
@@ -987,6 +1006,10 @@ int lbf_create(const lbf_config *cfg, lbf_sim **out) {
   AL(dalloc(s, &s->rlabel, N));
   AL(dalloc(s, &s->acc, 4));
   AL(dalloc(s, &s->counts, 4));
+  s->n_state_allocs = s->allocs.size();
+  // scratch, not part of a checkpoint
+  AL(dalloc(s, &s->rank, s->cap));
+  AL(dalloc(s, &s->rmlist, s->cap));
 #undef AL
   // zero everything that is read before being written
   auto zero = [&](void *p, size_t b) { return cudaMemsetAsync(p, 0, b, s->st); };
@@ -1047,7 +1070,6 @@ int lbf_create(const lbf_config *cfg, lbf_sim **out) {
     lbf_destroy(s);
     return fail(rc, msg);
   }
-  s->n_state_allocs = s->allocs.size();
   *out = s;
   return 0;
 }
@@ -1234,6 +1256,32 @@ size_t ckpt_bytes(const lbf_sim *s) {
   for (size_t k = 0; k < s->n_state_allocs; ++k) b += s->alloc_bytes[k];
   return b;
 }
+
+// the current labels and table in root order, as a full labelling leaves
+// them; the next step's patch starts from a full label copy
+int order_slots(lbf_sim *s) {
+  const int par = (int)(s->step & 1);
+  const Table &t = s->tab[par], &o = s->tab[1 - par];
+  const size_t cap = (size_t)s->cap;
+  s->ops->rank(make_params(s, s->step), s->st);
+  lbf::k_order_labels<<<s->list_blocks, 256, 0, s->st>>>(s->rank, s->label[par], s->N);
+  lbf::k_order_table<<<(s->cap + 255) / 256, 256, 0, s->st>>>(t, s->rank, o);
+  CK(cudaGetLastError());
+  int nb = 0;
+  CK(cudaMemcpyAsync(&nb, t.count, sizeof nb, cudaMemcpyDeviceToHost, s->st));
+  CK(cudaStreamSynchronize(s->st));
+  const size_t n = (size_t)std::min(nb, s->cap);
+  for (auto a : {&Table::m, &Table::p, &Table::V, &Table::dm})
+    CK(cudaMemcpyAsync(t.*a, o.*a, sizeof(double) * n, cudaMemcpyDeviceToDevice, s->st));
+  for (auto a : {&Table::id, &Table::atm, &Table::root, &Table::ng})
+    CK(cudaMemcpyAsync(t.*a, o.*a, sizeof(int) * n, cudaMemcpyDeviceToDevice, s->st));
+  CK(cudaMemsetAsync(o.V, 0, sizeof(double) * cap, s->st));
+  CK(cudaMemsetAsync(o.dm, 0, sizeof(double) * cap, s->st));
+  CK(cudaMemsetAsync(o.atm, 0, sizeof(int) * cap, s->st));
+  CK(cudaMemsetAsync(o.ng, 0, sizeof(int) * cap, s->st));
+  CK(cudaMemsetAsync(s->lab_full, 0xff, sizeof(int), s->st));
+  return 0;
+}
 }  // namespace
 
 int lbf_checkpoint_bytes(lbf_sim *s, size_t *bytes) {
@@ -1245,6 +1293,10 @@ int lbf_checkpoint_bytes(lbf_sim *s, size_t *bytes) {
 int lbf_checkpoint_save(lbf_sim *s, void *dst, size_t bytes) {
   if (!s || !dst) return fail(LBF_EINVAL, "NULL argument");
   if (bytes < ckpt_bytes(s)) return fail(LBF_EINVAL, "buffer smaller than lbf_checkpoint_bytes");
+  {
+    int rc = order_slots(s);
+    if (rc) return rc;
+  }
   CK(cudaStreamSynchronize(s->st));
   unsigned char *o = (unsigned char *)dst;
   CkptHeader h;
@@ -1330,7 +1382,7 @@ int lbf_bubbles(lbf_sim *s, lbf_bubble *out, int capacity, int *count) {
     if (rc) return rc;
     CK(cudaMallocHost((void **)&s->bub_host, 16 + sizeof(lbf_bubble) * (size_t)s->cap));
   }
-  lbf::pack_bubbles_launch(s->tab[s->step & 1], s->bub_dev, rows, s->st);
+  lbf::pack_bubbles_launch(s->tab[s->step & 1], s->bub_dev, rows, s->cap, s->st);
   CK(cudaGetLastError());
   // the header and the first rows in one copy; the rest only when present
   constexpr int kFirst = 64;
@@ -1358,27 +1410,33 @@ int lbf_fields(lbf_sim *s, unsigned mask, void *const *dst, int dst_is_device, i
   Params p = make_params(s, s->step);
   p.label_new = s->label[par];
   const size_t N = (size_t)s->N;
+  void *out[11] = {nullptr};
   int k = 0;
   for (int bit = 0; bit < 11; ++bit) {
     if (!(mask & (1u << bit))) continue;
-    void *out = dst[k++];
-    if (!out) return fail(LBF_EINVAL, "NULL destination");
+    out[bit] = dst[k++];
+    if (!out[bit]) return fail(LBF_EINVAL, "NULL destination");
+  }
+  if (dst_is_device) {
+    if (mask) s->ops->fields(p, par, mask, out, dtype, s->st);
+    CK(cudaGetLastError());
+    return 0;
+  }
+  for (int bit = 0; bit < 11; ++bit) {
+    if (!(mask & (1u << bit))) continue;
     const bool is_int = bit == FLD_FLAGS || bit == FLD_LABEL;
     const int width = (bit == FLD_U || bit == FLD_NORMAL) ? 3 : 1;
     const size_t bytes = N * width * (is_int ? 4 : (dtype ? 8 : 4));
-    if (dst_is_device) {
-      s->ops->field(p, par, bit, out, dtype, s->st);
-      CK(cudaGetLastError());
-    } else {
-      if (!s->staging) {
-        int rc = dev_alloc(s, &s->staging, N * 3 * 8);
-        if (rc) return rc;
-      }
-      s->ops->field(p, par, bit, s->staging, dtype, s->st);
-      CK(cudaGetLastError());
-      int rc = copy_to_host(s, out, s->staging, bytes);
+    if (!s->staging) {
+      int rc = dev_alloc(s, &s->staging, N * 3 * 8);
       if (rc) return rc;
     }
+    void *one[11] = {nullptr};
+    one[bit] = s->staging;
+    s->ops->fields(p, par, 1u << bit, one, dtype, s->st);
+    CK(cudaGetLastError());
+    int rc = copy_to_host(s, out[bit], s->staging, bytes);
+    if (rc) return rc;
   }
   return 0;
 }

@@ -104,6 +104,10 @@ struct Table {
   double *m, *p, *V, *dm;  // gas mass, pressure, volume, gas gained this step
   int *id, *atm, *root;    // stable id, atmosphere flag, canonical label
   int *ng;                 // gas cells of the bubble (V = ng + interface shares)
+  // Rows are slots: the labels of cells hold slot numbers, which stay as
+  // they are while patched steps move roots past one another.  A bubble's
+  // public number is the rank of its root among all roots (k_rank); a full
+  // labelling numbers the slots in that order again.
   int *count;              // number of rows (device)
 };
 
@@ -157,9 +161,9 @@ struct Params {
   // from outside (full labelling).  NULL means always full.
   int *gas_dirty;
   uint8_t *tdirty;  // per union-find tile: touched by added gas cells since the last forest update
-  // set by the marking when an added gas cell could join two bubbles or
-  // move a bubble's smallest cell index: the step then needs the full
-  // labelling (else the labels of the last step, patched, are exact)
+  // set by the labelling check when a conversion could join, split, empty or
+  // begin a bubble: the step then needs the full labelling (else the labels
+  // of the last step, patched, are exact)
   int *lab_slow;
   // after steps labelled without the union-find: bit 0, gas cells were
   // added (the forest lags behind in the touched tiles, tdirty, which the
@@ -175,10 +179,11 @@ struct Params {
   // state was set from outside): the next patched labelling then starts
   // from a full copy instead of copying the listed cells
   int *lab_full;
-  // root moves of a patched step: [0] the bubble whose root cell turns
-  // interface (-1 none; one bubble per step), [1] set when some bubble's
-  // root is lowered by an added gas cell
-  int *rmv;
+  // root moves of a patched step: [0] the number of bubbles whose root cell
+  // turns interface (listed in rmlist), less one, [1] the blocks of the root
+  // scan that are done
+  int *rmv, *rmlist;
+  int *rank;  // scratch of exports: the public number of each slot
   int tile_blocks;  // grid of the tile loops of the union-find (two blocks per SM)
   // label of each current root cell (rank among the sorted roots, -1 past
   // the bubble capacity); read only at cells that are roots
@@ -454,6 +459,21 @@ __device__ __forceinline__ void agg_add(double *base, int key, double v, double 
     atomicAdd(base + key, s);
   }
   __syncwarp();
+}
+
+// how many of cnt roots are smaller than `mine`: every thread of the block
+// takes part, the roots staged 1024 at a time through sr
+__device__ __forceinline__ int count_below(const int *root, int cnt, int mine, int *sr) {
+  int r = 0;
+  for (int j0 = 0; j0 < cnt; j0 += 1024) {
+    const int m = min(1024, cnt - j0);
+    __syncthreads();
+    for (int j = threadIdx.x; j < m; j += blockDim.x) sr[j] = root[j0 + j];
+    __syncthreads();
+#pragma unroll 8
+    for (int j = 0; j < m; ++j) r += sr[j] < mine;
+  }
+  return r;
 }
 
 }  // namespace lbf

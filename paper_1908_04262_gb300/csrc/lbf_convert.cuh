@@ -173,13 +173,11 @@ __device__ __forceinline__ long long list_cell(const Params &p, int k, int nm) {
 }
 
 // An added gas cell (an emptied interface cell) keeps the bubble structure
-// of the last labelling when it carries a bubble label L (the smallest of
-// its gas neighbours' as an interface cell), every gas neighbour after the
+// of the last labelling when it carries a bubble label L (that of one of
+// its gas neighbours as an interface cell), every gas neighbour after the
 // conversion carries L (it joins no other bubble) and one of them is a gas
 // cell of the last step that stays gas (it is joined to its bubble).  Below
-// the bubble's root it becomes the new root (the patch takes the minimum);
-// the labels, ranks of the roots, stay as they are while it lies above the
-// root of bubble L - 1.
+// the bubble's root it becomes the new root.
 template <int D>
 __device__ __forceinline__ bool addition_keeps_bubble(const Params &p, const Cell &c, int n) {
   const int L = p.label_old[n];
@@ -192,8 +190,8 @@ __device__ __forceinline__ bool addition_keeps_bubble(const Params &p, const Cel
     fn[i] = p.flags[m];
     ln[i] = p.label_old[m];
   }
-  if (L < 0 || (n < p.told.root[L] && L > 0 && n < p.told.root[L - 1])) return false;
-  if (n < p.told.root[L]) p.rmv[1] = 1;
+  if (L < 0) return false;
+  if (n < p.told.root[L]) atomicMin(p.tnew.root + L, n);
   bool anchored = false;
 #pragma unroll
   for (int i = 1; i < Lat<D>::Q; ++i) {
@@ -222,11 +220,8 @@ __device__ __forceinline__ bool removal_keeps_bubble(const Params &p, const Cell
   constexpr int NS = D == 3 ? 27 : 9, CTR = D == 3 ? 13 : 4;
   const int L = p.label_old[n];
   if (L < 0) return false;
-  if (n == p.told.root[L]) {
-    // the root moves up: k_root_scan finds the new one (one bubble per step)
-    const int prev = atomicCAS(p.rmv, -1, L);
-    if (prev != -1 && prev != L) return false;
-  }
+  // the root moves up: k_root_scan finds the new one
+  if (n == p.told.root[L]) p.rmlist[atomicAdd(p.rmv, 1) + 1] = L;
   if (p.atmosphere && (D == 2 ? c.y : c.z) == p.top_layer) return false;
   unsigned gas = 0, link = 0, gone = 0;  // bit k: stencil cell k is gas after the conversion /
                                          // a gas neighbour of the centre / linked and turning interface
@@ -265,53 +260,105 @@ __device__ __forceinline__ bool removal_keeps_bubble(const Params &p, const Cell
   return (link & ~reach) == 0;
 }
 
-// After the labelling check, when a bubble's root cell turns interface: its
-// new root is the smallest cell after the old one that is gas after the
-// conversion and carries the bubble's label (a gas cell that stays, or an
-// emptied interface cell of the bubble).  One block scans forward 8 cells
-// per thread at a time, at most four times; the labels (ranks of the roots)
-// stay valid when the new root lies below the next bubble's and no root was
-// lowered in the same step, otherwise (or when the scan gives up) the step
+// After the labelling check: the new root of every bubble whose root cell
+// turns interface.  Unless a cell added below the old root took its place,
+// it is the smallest cell after the old one that is gas after the conversion
+// and carries the bubble's label (a gas cell that stays, or an emptied
+// interface cell of the bubble).  The removed root kept a gas neighbour of
+// its bubble, and none lies in a lower plane (row in 2D), so the new root
+// lies in the old one's plane or the next, unless the bubble is joined
+// across the periodic face there: then the scan finds nothing and the step
 // takes the full labelling.
-static __global__ void __launch_bounds__(1024) k_root_scan(Params p) {
-  __shared__ int L, found;
-  if (threadIdx.x == 0) {
-    L = p.rmv[0];
-    found = 0x7fffffff;
-  }
-  __syncthreads();
-  if (L < 0) {
-    if (threadIdx.x == 0) p.rmv[1] = 0;
-    return;
-  }
-  const long long r0 = (long long)p.told.root[L] + 1;
-  for (int it = 0; it < 4; ++it) {
-    const long long base = r0 + (long long)it * (8 * 1024) + 8 * (long long)threadIdx.x;
+//
+// A block per bubble; latency-bound: in nearly every case the first round
+// (64 KB of flags in 16-byte loads, labels read at gas cells only) finds it.
+// Reaching to the end of the next plane, for any number of bubbles a step
+// (the limits had been 32,768 cells and one bubble), is one of the two things
+// that keep large foams on the patched labelling: see label_fast.
+//
+// The last block to finish writes the step's choice of labelling branch,
+// lab_fast: patched unless the state was set from outside (gas_dirty -1) or
+// a conversion was refused (lab_slow).
+constexpr int SCAN_THREADS = 512, SCAN_WORDS = 8, SCAN_BLOCKS = 32;
+template <int D>
+__global__ void __launch_bounds__(SCAN_THREADS) k_root_scan(Params p) {
+  __shared__ int found;
+  const int cnt = p.rmv[0] + 1;
+  const long long layer = D == 3 ? (long long)p.nx * p.ny : p.nx;
+  for (int e = blockIdx.x; e < cnt; e += gridDim.x) {
+    const int L = p.rmlist[e];
+    const long long r0 = p.told.root[L];
+    if (p.tnew.root[L] < r0) continue;  // the same for every thread
+    const long long end = min(p.N, (r0 / layer + 2) * layer);
+    if (threadIdx.x == 0) found = 0x7fffffff;
+    __syncthreads();
+    // (the flag array's allocation is 16-byte aligned and holds N bytes: a
+    // word that reaches past N is read bytewise)
+    for (long long base = (r0 + 1) & ~15ll; base < end; base += 16ll * SCAN_WORDS * SCAN_THREADS) {
+      unsigned w[SCAN_WORDS][4];
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const long long n = base + j;
-      if (n < p.N && post_type(p.flags[n]) == T_GAS && p.label_old[n] == L) atomicMin(&found, (int)n);
+      for (int j = 0; j < SCAN_WORDS; ++j) {
+        const long long n0 = base + 16ll * (j * SCAN_THREADS + (int)threadIdx.x);
+        if (n0 + 16 <= p.N) {
+          const uint4 v = *reinterpret_cast<const uint4 *>(p.flags + n0);
+          w[j][0] = v.x;
+          w[j][1] = v.y;
+          w[j][2] = v.z;
+          w[j][3] = v.w;
+        } else {
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            w[j][q] = 0;
+#pragma unroll
+            for (int b = 0; b < 4; ++b)
+              w[j][q] |= (unsigned)(n0 + 4 * q + b < p.N ? p.flags[n0 + 4 * q + b] : (uint8_t)T_WALL) << (8 * b);
+          }
+        }
+      }
+#pragma unroll
+      for (int j = 0; j < SCAN_WORDS; ++j) {
+        // sixteen liquid cells without marks
+        if (((w[j][0] & w[j][1] & w[j][2] & w[j][3]) & 0x01010101u) == 0x01010101u &&
+            ((w[j][0] | w[j][1] | w[j][2] | w[j][3]) & 0x1e1e1e1eu) == 0u)
+          continue;
+        const long long n0 = base + 16ll * (j * SCAN_THREADS + (int)threadIdx.x);
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          for (int b = 0; b < 4; ++b) {
+            const long long n = n0 + 4 * q + b;
+            if (post_type((uint8_t)(w[j][q] >> (8 * b))) == T_GAS && n > r0 && n < end && p.label_old[n] == L)
+              atomicMin(&found, (int)n);
+          }
+      }
+      __syncthreads();
+      const bool done = found != 0x7fffffff;
+      __syncthreads();
+      if (done) break;
+    }
+    if (threadIdx.x == 0) {
+      if (found == 0x7fffffff) {
+        atomicOr(p.lab_slow, 1);
+      } else {
+        p.tnew.root[L] = found;
+      }
     }
     __syncthreads();
-    const bool done = found != 0x7fffffff;
-    __syncthreads();
-    if (done) break;
   }
   if (threadIdx.x == 0) {
-    const int nb = *p.told.count;
-    if (found == 0x7fffffff || p.rmv[1] || (L + 1 < nb && found > p.told.root[L + 1]))
-      atomicOr(p.lab_slow, 1);
-    else
-      p.tnew.root[L] = found;
-    p.rmv[0] = -1;
-    p.rmv[1] = 0;
+    __threadfence();
+    if (atomicAdd(p.rmv + 1, 1) == (int)gridDim.x - 1) {
+      __threadfence();
+      const bool fast = *p.gas_dirty >= 0 && __ldcg(p.lab_slow) == 0;
+      *p.lab_fast = fast;
+      *p.lab_full = !fast;
+    }
   }
 }
 
 // after the marking (every mark final): the emptied cells are on the marked
 // list, the gas cells turned interface on the new-interface list; any of
-// them that could join, split, empty or re-root a bubble vetoes the patched
-// labelling of this step (lab_slow)
+// them that could join, split or empty a bubble vetoes the patched labelling
+// of this step (lab_slow); root moves are recorded
 template <int D>
 __global__ void __launch_bounds__(128) k_label_check(Params p) {
   const int nm = *p.mcount, total = nm + *p.ncount;
@@ -669,51 +716,63 @@ __global__ void k_nucleate(Params p, int par, double cx, double cy, double cz, d
 // ---------------------------------------------------------------------------
 // export and ledgers
 
+// rank[k]: the public number of slot k, the count of smaller roots
+constexpr int RANK_THREADS = 128;
+static __global__ void __launch_bounds__(RANK_THREADS) k_rank(const int *root, const int *count, int *rank) {
+  __shared__ int sr[1024];
+  const int cnt = *count;
+  for (int k0 = blockIdx.x * RANK_THREADS; k0 < cnt; k0 += gridDim.x * RANK_THREADS) {
+    const int k = k0 + (int)threadIdx.x;
+    const int r = count_below(root, cnt, k < cnt ? root[k] : 0, sr);
+    if (k < cnt) rank[k] = r;
+  }
+}
+
+// The fields of `mask` in one pass, so that the populations are read once
+// whichever of density, velocity and mass are asked for.  Bound by HBM: at
+// 256^3 in shifted FP16 (rho, u, alpha, flags, conc, label) one launch per
+// field moved the populations three times; a 32^3 lattice paid six launches.
+struct FieldPtrs {
+  void *p[11];  // by field bit
+};
 template <int D, class S>
-__global__ void k_fields(Params p, int par, int which, void *out, int dtype) {
+__global__ void k_fields(Params p, int par, unsigned mask, FieldPtrs out, int dtype) {
   using R = typename ST<S>::R;
   Cell c;
   if (!grid_cell(p, c)) return;
   const long long n = c.n;
   const int t = ftype(p.flags[n]);
   const bool fluid = t == T_LIQ || t == T_IFC;
-  double v[3] = {0.0, 0.0, 0.0};
-  int width = 1;
-  switch (which) {
-    case FLD_RHO: if (fluid) v[0] = (double)sum_out_f<D, S>(p, c, n, par, nullptr); break;
-    case FLD_U:
-      width = 3;
-      if (fluid) {
-        R u[3];
-        sum_out_f<D, S>(p, c, n, par, u);
-        v[0] = u[0]; v[1] = u[1]; v[2] = u[2];
-      }
-      break;
-    case FLD_ALPHA: v[0] = (double)((const R *)p.phi)[n]; break;
-    case FLD_MASS:
-      if (t == T_IFC) v[0] = (double)((const R *)p.M)[n];
-      else if (t == T_LIQ) v[0] = (double)sum_out_f<D, S>(p, c, n, par, nullptr);
-      break;
-    case FLD_CONC: if (fluid) v[0] = (double)sum_out_g<D, S>(p, c, n, par); break;
-    case FLD_KAPPA: if (t == T_IFC) v[0] = (double)((const R *)p.kappa)[n]; break;
-    case FLD_PI: if (t == T_IFC) v[0] = (double)((const R *)p.Pi)[n]; break;
-    case FLD_DSTAR: if (t == T_IFC) v[0] = (double)((const R *)p.dst)[n]; break;
-    case FLD_NORMAL:
-      width = 3;
-      if (t == T_IFC) {
-        const R *nr = (const R *)p.nrm;
-        v[0] = nr[n]; v[1] = nr[p.N + n]; v[2] = nr[2 * p.N + n];
-      }
-      break;
-    case FLD_FLAGS: ((int *)out)[n] = t; return;
-    case FLD_LABEL: ((int *)out)[n] = (t == T_GAS || t == T_IFC) ? p.label_new[n] : -1; return;
-  }
-  for (int k = 0; k < width; ++k) {
+  auto want = [&](int f) { return ((mask >> f) & 1u) != 0; };
+  auto put = [&](int f, long long k, double v) {
     if (dtype == 1)
-      ((double *)out)[width * n + k] = v[k];
+      ((double *)out.p[f])[k] = v;
     else
-      ((float *)out)[width * n + k] = (float)v[k];
+      ((float *)out.p[f])[k] = (float)v;
+  };
+  double rho = 0.0;
+  R u[3] = {0, 0, 0};
+  if (fluid && (want(FLD_RHO) || want(FLD_U) || (want(FLD_MASS) && t == T_LIQ)))
+    rho = (double)sum_out_f<D, S>(p, c, n, par, u);
+  if (want(FLD_RHO)) put(FLD_RHO, n, rho);
+  if (want(FLD_U))
+    for (int k = 0; k < 3; ++k) put(FLD_U, 3 * n + k, (double)u[k]);
+  if (want(FLD_ALPHA)) put(FLD_ALPHA, n, (double)((const R *)p.phi)[n]);
+  if (want(FLD_MASS)) put(FLD_MASS, n, t == T_IFC ? (double)((const R *)p.M)[n] : (t == T_LIQ ? rho : 0.0));
+  if (want(FLD_FLAGS)) ((int *)out.p[FLD_FLAGS])[n] = t;
+  if (want(FLD_CONC)) put(FLD_CONC, n, fluid ? (double)sum_out_g<D, S>(p, c, n, par) : 0.0);
+  const bool ifc = t == T_IFC;
+  if (want(FLD_KAPPA)) put(FLD_KAPPA, n, ifc ? (double)((const R *)p.kappa)[n] : 0.0);
+  if (want(FLD_LABEL)) {
+    const int l = (t == T_GAS || ifc) ? p.label_new[n] : -1;
+    ((int *)out.p[FLD_LABEL])[n] = l >= 0 ? p.rank[l] : -1;
   }
+  if (want(FLD_PI)) put(FLD_PI, n, ifc ? (double)((const R *)p.Pi)[n] : 0.0);
+  if (want(FLD_NORMAL)) {
+    const R *nr = (const R *)p.nrm;
+    for (int k = 0; k < 3; ++k) put(FLD_NORMAL, 3 * n + k, ifc ? (double)nr[k * p.N + n] : 0.0);
+  }
+  if (want(FLD_DSTAR)) put(FLD_DSTAR, n, ifc ? (double)((const R *)p.dst)[n] : 0.0);
 }
 
 // [0] liquid mass, [1] dissolved gas, [2] non-finite populations, plus cell

@@ -6,8 +6,8 @@
 // Gas cells connected over lattice links (D2Q9: 8 neighbours, D3Q19: 18)
 // form a bubble.  A lock-free union-find links every root under the smaller
 // index, so the root of a component is its smallest linear cell index; the
-// bubbles are numbered in the order of those roots.  Interface cells join the
-// bubble of their gas neighbour with the smallest number.  Old and new
+// bubbles are numbered in the order of those roots (k_rank).  Interface
+// cells join the bubble of their gas neighbour with the smallest number.  Old and new
 // bubbles that share gas or interface cells form groups; within a group the
 // old gas content is split over the new bubbles in proportion to volume.
 #pragma once
@@ -498,62 +498,66 @@ __device__ __forceinline__ void hash_insert(const Params &p, unsigned long long 
   atomicOr(p.err, ERR_HASH);
 }
 
-// new labels, volumes, atmosphere flags and old->new overlap pairs
+// new labels, volumes, atmosphere flags and old->new overlap pairs: one warp
+// per 32-cell segment along x, one lane per cell
 template <int D, class R>
-__global__ void __launch_bounds__(256) k_relabel(Params p) {
-  __shared__ double wbuf[256];
-  if (label_fast(p)) return;
-  // row blocks of blockDim.x cells along x, walked by a grid of any size
-  const int nbx = (p.nx + (int)blockDim.x - 1) / (int)blockDim.x;
-  const int nrb = nbx * p.ny * p.nz;
-  for (int rb = block_id(); rb < nrb; rb += block_count()) {
-  const int yz = rb / nbx, xb = (rb - yz * nbx) * (int)blockDim.x + (int)threadIdx.x;
-  Cell c = cell_at(p, xb < p.nx ? xb : p.nx - 1, yz % p.ny, yz / p.ny);
-  const bool inr = xb < p.nx;
-  const long long n = c.n;
-  const uint8_t fl = inr ? p.flags[n] : (uint8_t)T_WALL;
-  const int t = post_type(fl);
-  int knew = -1, ngas = 0;
-  double v = 0.0;
-  if (t == T_GAS) {
-    knew = p.rlabel[p.parent[n]];
-    ngas = p.lsize[n];  // non-zero only at tile-local roots
-    if (p.atmosphere && knew >= 0 && (D == 2 ? c.y : c.z) == p.top_layer && !p.tnew.atm[knew]) p.tnew.atm[knew] = 1;
-  } else if (t == T_IFC) {
+__device__ __forceinline__ void relabel_all(const Params &p, double *wbuf) {
+  const int lane = threadIdx.x & 31;
+  const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nwarps = (gridDim.x * blockDim.x) >> 5;
+  const int nseg = ((p.nx + 31) >> 5) * p.ny * p.nz;
+  for (int seg = warp; seg < nseg; seg += nwarps) {
+    Cell c;
+    const bool inr = seg_cell(p, seg, lane, c);
+    const long long n = c.n;
+    const uint8_t fl = inr ? p.flags[n] : (uint8_t)T_WALL;
+    const int t = post_type(fl);
+    int knew = -1, ngas = 0;
+    double v = 0.0;
+    if (t == T_GAS) {
+      knew = p.rlabel[p.parent[n]];
+      ngas = p.lsize[n];  // non-zero only at tile-local roots
+      if (p.atmosphere && knew >= 0 && (D == 2 ? c.y : c.z) == p.top_layer && !p.tnew.atm[knew]) p.tnew.atm[knew] = 1;
+    } else if (t == T_IFC) {
 #pragma unroll
-    for (int i = 1; i < Lat<D>::Q; ++i) {
-      const long long m = nb<D>(p, c, i);
-      if (post_type(p.flags[m]) == T_GAS) {
-        const int k = p.rlabel[p.parent[m]];
-        if (k >= 0 && (knew < 0 || k < knew)) knew = k;
+      for (int i = 1; i < Lat<D>::Q; ++i) {
+        const long long m = nb<D>(p, c, i);
+        if (post_type(p.flags[m]) == T_GAS) {
+          const int k = p.rlabel[p.parent[m]];
+          if (k >= 0 && (knew < 0 || k < knew)) knew = k;
+        }
       }
+      if (knew >= 0) v = 1.0 - (double)((const R *)p.phi)[n];
     }
-    if (knew >= 0) v = 1.0 - (double)((const R *)p.phi)[n];
-  }
-  if (inr) p.label_new[n] = knew;
-  // gas cells are counted (the bubble update adds them to the volume),
-  // interface cells add their gas share 1 - alpha
-  const bool gcontrib = knew >= 0 && ngas != 0;
-  if (__any_sync(0xffffffffu, gcontrib)) agg_count(p.tnew.ng, gcontrib ? knew : -1, ngas);
-  const bool contrib = knew >= 0 && v != 0.0;
-  if (__any_sync(0xffffffffu, contrib)) agg_add(p.tnew.V, contrib ? knew : -1, v, wbuf + (threadIdx.x & ~31));
-  // old -> new overlap pairs (cells without a new label have none: no
-  // old label read, and warps without any pair skip the match)
-  const int kold = (inr && knew >= 0) ? p.label_old[n] : -1;
-  const bool pair = kold >= 0 && knew >= 0;
-  if (!__any_sync(0xffffffffu, pair)) continue;
-  const unsigned long long key = pair ? (((unsigned long long)kold << 32) | (unsigned)knew) : HASH_EMPTY;
-  const unsigned peers = __match_any_sync(0xffffffffu, key);
-  if (pair && (threadIdx.x & 31) == __ffs(peers) - 1) hash_insert(p, key);
+    if (inr) p.label_new[n] = knew;
+    // gas cells are counted (the bubble update adds them to the volume),
+    // interface cells add their gas share 1 - alpha
+    const bool gcontrib = knew >= 0 && ngas != 0;
+    if (__any_sync(0xffffffffu, gcontrib)) agg_count(p.tnew.ng, gcontrib ? knew : -1, ngas);
+    const bool contrib = knew >= 0 && v != 0.0;
+    if (__any_sync(0xffffffffu, contrib)) agg_add(p.tnew.V, contrib ? knew : -1, v, wbuf);
+    // old -> new overlap pairs (cells without a new label have none: no
+    // old label read, and warps without any pair skip the match)
+    const int kold = (inr && knew >= 0) ? p.label_old[n] : -1;
+    const bool pair = kold >= 0 && knew >= 0;
+    if (!__any_sync(0xffffffffu, pair)) continue;
+    const unsigned long long key = pair ? (((unsigned long long)kold << 32) | (unsigned)knew) : HASH_EMPTY;
+    const unsigned peers = __match_any_sync(0xffffffffu, key);
+    if (pair && lane == __ffs(peers) - 1) hash_insert(p, key);
   }
 }
 
-// one block of 1024 threads: carry gas content from the old to the new table.
+// one block of 1024 threads: carry gas content from the old to the new table
+// (a patched step has its own short form, update_kept, in the same launch:
+// as two kernels the one not needed cost 2.7 us of the step's chain).
 // Group bookkeeping lives in shared memory when there are at most
 // K10_SMEM old + new bubbles, in the global scratch arrays otherwise.
 constexpr int K10_SMEM = 512;
+static __device__ __forceinline__ void update_kept(const Params &p);
 static __global__ void __launch_bounds__(1024) k_bubble_update(Params p) {
-  if (label_fast(p)) return;
+  if (label_fast(p)) {
+    update_kept(p);
+    return;
+  }
   __shared__ int sfresh[1024];
   __shared__ int sbase;
   __shared__ int s_par[K10_SMEM], s_nold[K10_SMEM], s_nnew[K10_SMEM], s_atm[K10_SMEM], s_minid[K10_SMEM],
@@ -697,24 +701,26 @@ static __global__ void __launch_bounds__(1024) k_bubble_update(Params p) {
 }
 
 // ---------------------------------------------------------------------------
-// Labelling of a step whose conversion kept every bubble's cells, number and
-// root: added gas cells touch no gas cell of another bubble and lie above
-// their bubble's root (checked by the marking), removed gas cells leave
-// their bubble connected (k_label_check); otherwise lab_slow is set.  Every
-// bubble keeps its cells, its number and its root, so the labels of the last
-// step stand except at the filled cells (-1), the added gas cells (the label
-// they had as interface cells, which is their bubble's) and the interface
-// cells after the conversion (smallest label of their gas neighbours).  The
-// result equals the full labelling's.  The step graph picks this branch or
-// the full one on the device: k_label_choose sets lab_fast, and the kernels
-// of the branch not taken return at once.
-static __global__ void k_label_choose(Params p) {
-  const int d = *p.gas_dirty;  // -1: the state was set from outside
-  const bool fast = d >= 0 && *p.lab_slow == 0;
-  *p.lab_fast = fast;
-  *p.lab_full = !fast;
-  *p.lab_slow = 0;
-}
+// Labelling of a step whose conversion kept every bubble's cells: added gas
+// cells touch no gas cell of another bubble, removed gas cells leave their
+// bubble connected (k_label_check); otherwise lab_slow is set.  The labels
+// (slots) of the last step then stand except at the filled cells (-1), the
+// added gas cells (the label they had as interface cells, which is their
+// bubble's) and the interface cells after the conversion (the gas neighbour
+// whose bubble has the smallest root).  Root cells move as bubbles grow and
+// deform; the labels do not change with them.  The result equals the full
+// labelling's once slots are read through their ranks.  The step graph picks
+// this branch or the full one on the device (k_root_scan writes lab_fast):
+// the union-find kernels return at once, the others take the branch inside.
+//
+// Why slots: with the labels themselves in root order, every root that moved
+// past another's, and every second root moved in a step, forced a full
+// labelling.  In foams of a few hundred bubbles that is nearly every step
+// (256^3 with 200 bubbles 1,262 steps of 1,336, 512x512x384 with 2,000 all
+// of them), while in the same runs one step in a thousand joined or split
+// bubbles.  Measured, ms for the timed passes of those foams: 256^3 shifted
+// FP16, 8 steps, 9.86 -> 6.61; 512x512x384 shifted BF16, 4 steps, 31.0 ->
+// 20.0; 2D 450x650, 150 bubbles, 20 steps, 1.76 -> 1.31.
 
 // At the start of a step, before its marking: bring label_new (the labels
 // of the step before last) up to the last labels wherever they differ.
@@ -725,10 +731,15 @@ static __global__ void k_label_choose(Params p) {
 // own cells; a full labelling overwrites every label.
 static __global__ void k_label_sync(Params p) {
   const long long tid = blockIdx.x * (long long)blockDim.x + threadIdx.x, nt = (long long)gridDim.x * blockDim.x;
-  // the roots of the next table start from the last ones (a patched step
-  // lowers a bubble's root to the gas cells it adds below it)
+  // the roots of the next table start from the last ones (the labelling
+  // check moves them); the check's findings are cleared
   const int nbub = *p.told.count;
   for (long long k = tid; k < nbub; k += nt) p.tnew.root[k] = p.told.root[k];
+  if (tid == 0) {
+    *p.lab_slow = 0;
+    p.rmv[0] = -1;
+    p.rmv[1] = 0;
+  }
   if (*p.lab_full) {
     const long long n4 = p.N >> 2;
     const int4 *src = reinterpret_cast<const int4 *>(p.label_old);
@@ -748,9 +759,7 @@ static __global__ void k_label_sync(Params p) {
 // cell, then per interface cell after the conversion; gas counts grow by the
 // added cells; volumes collect the interface shares 1 - alpha.
 template <int D, class R>
-__global__ void __launch_bounds__(128) k_label_fast(Params p) {
-  __shared__ double wbuf[128];
-  if (!label_fast(p)) return;
+__device__ __forceinline__ void patch_labels(const Params &p, double *wbuf) {
   const int nbub = *p.told.count, nm = *p.mcount, ni = *p.inext_count, nn = *p.ncount;
   const int tid = blockIdx.x * blockDim.x + threadIdx.x, nthreads = gridDim.x * blockDim.x;
   if (tid == 0) {
@@ -784,7 +793,6 @@ __global__ void __launch_bounds__(128) k_label_fast(Params p) {
         p.label_new[n] = -1;
       } else if (t == T_GAS) {
         kg = p.label_old[n];
-        if (kg >= 0) atomicMin(p.tnew.root + kg, n);
         if (p.atmosphere && kg >= 0) {
           const Cell c = make_cell(p, n);
           if ((D == 2 ? c.y : c.z) == p.top_layer) p.tnew.atm[kg] = 1;
@@ -807,7 +815,8 @@ __global__ void __launch_bounds__(128) k_label_fast(Params p) {
       for (int i = 1; i < Lat<D>::Q; ++i) {
         if (post_type(fn[i]) == T_GAS) {
           const int l = ln[i];
-          if (l >= 0 && (knew < 0 || l < knew)) knew = l;
+          if (l < 0 || l == knew) continue;
+          if (knew < 0 || p.tnew.root[l] < p.tnew.root[knew]) knew = l;
         }
       }
       p.label_new[n] = knew;
@@ -817,18 +826,27 @@ __global__ void __launch_bounds__(128) k_label_fast(Params p) {
       }
     }
     if (__any_sync(0xffffffffu, kg >= 0)) agg_count(p.tnew.ng, kg, dg);
-    if (__any_sync(0xffffffffu, kv >= 0)) agg_add(p.tnew.V, kv, v, wbuf + (threadIdx.x & ~31));
+    if (__any_sync(0xffffffffu, kv >= 0)) agg_add(p.tnew.V, kv, v, wbuf);
   }
 }
 
+// the new labels of a step by the branch chosen, in one launch
+template <int D, class R>
+__global__ void __launch_bounds__(128) k_relabel(Params p) {
+  __shared__ double wbuf[128];
+  if (label_fast(p))
+    patch_labels<D, R>(p, wbuf + (threadIdx.x & ~31));
+  else
+    relabel_all<D, R>(p, wbuf + (threadIdx.x & ~31));
+}
+
 // the bubble update of such a step: every group is one old and one new
-// bubble with the same number, so each bubble keeps its id and gas (plus the
+// bubble in the same slot, so each bubble keeps its id and gas (plus the
 // flux of this step); the arithmetic is the general update's for such a
 // group.  One thread per bubble.
-static __global__ void k_bubble_update_fast(Params p) {
-  if (!label_fast(p)) return;
+static __device__ __forceinline__ void update_kept(const Params &p) {
   const int nbub = *p.tnew.count;
-  const int tid = blockIdx.x * blockDim.x + threadIdx.x, nt = gridDim.x * blockDim.x;
+  const int tid = threadIdx.x, nt = blockDim.x;
   for (int k = tid; k < nbub; k += nt) {
     const double mold = p.told.m[k] + p.told.dm[k];
     p.told.m[k] = mold;

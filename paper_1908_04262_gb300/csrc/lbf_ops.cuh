@@ -117,25 +117,16 @@ struct OpsImpl final : Ops {
     k_sort_roots<<<1, 1024, P * sizeof(int), s>>>(p);
   }
   void label_relabel(const Params &p, cudaStream_t s) override {
-    // row blocks walked by a grid of 16 blocks per SM
-    const unsigned nrb = row_grid(p).x * (unsigned)p.ny * (unsigned)p.nz;
-    const unsigned g = (unsigned)p.warp_blocks < nrb ? (unsigned)p.warp_blocks : nrb;
-    k_relabel<D, R><<<g, row_block(p), 0, s>>>(p);
+    // four blocks per SM for the patch's short lists; the full relabelling
+    // walks every segment of the lattice with them
+    k_relabel<D, R><<<p.list_blocks, 128, 0, s>>>(p);
   }
   void bubble_update(const Params &p, cudaStream_t s) override { k_bubble_update<<<1, 1024, 0, s>>>(p); }
   void label_check(const Params &p, cudaStream_t s) override {
     k_label_check<D><<<p.list_blocks, 128, 0, s>>>(p);
-    k_root_scan<<<1, 1024, 0, s>>>(p);
+    k_root_scan<D><<<SCAN_BLOCKS, SCAN_THREADS, 0, s>>>(p);
   }
-  void label_choose(const Params &p, cudaStream_t s) override { k_label_choose<<<1, 1, 0, s>>>(p); }
   void label_sync(const Params &p, cudaStream_t s) override { k_label_sync<<<p.list_blocks, 128, 0, s>>>(p); }
-  void label_fast(const Params &p, cudaStream_t s) override {
-    k_label_fast<D, R><<<p.list_blocks, 128, 0, s>>>(p);
-  }
-  void bubble_update_fast(const Params &p, cudaStream_t s) override {
-    const unsigned g = blocks_for(p.cap, 128);
-    k_bubble_update_fast<<<g < (unsigned)p.list_blocks ? g : (unsigned)p.list_blocks, 128, 0, s>>>(p);
-  }
   void geometry(const Params &p, cudaStream_t s) override {
     k_geometry<D, R><<<p.warp_blocks, 128, 0, s>>>(p);
     if (p.kappa_hf) k_hf_kappa<D, R><<<p.list_blocks, 128, 0, s>>>(p);
@@ -153,8 +144,14 @@ struct OpsImpl final : Ops {
   void disjoining(const Params &p, cudaStream_t s) override {
     k_disjoining<D, R><<<p.list_blocks, 128, 0, s>>>(p);
   }
-  void field(const Params &p, int par, int which, void *out, int dtype, cudaStream_t s) override {
-    k_fields<D, S><<<row_grid(p), row_block(p), 0, s>>>(p, par, which, out, dtype);
+  void rank(const Params &p, cudaStream_t s) override {
+    k_rank<<<blocks_for(p.cap, RANK_THREADS), RANK_THREADS, 0, s>>>(p.told.root, p.told.count, p.rank);
+  }
+  void fields(const Params &p, int par, unsigned mask, void *const (&out)[11], int dtype, cudaStream_t s) override {
+    FieldPtrs f;
+    for (int k = 0; k < 11; ++k) f.p[k] = out[k];
+    if (mask >> FLD_LABEL & 1u) rank(p, s);
+    k_fields<D, S><<<row_grid(p), row_block(p), 0, s>>>(p, par, mask, f, dtype);
   }
   void ledger(const Params &p, int par, double *acc, unsigned long long *counts, cudaStream_t s) override {
     k_ledger<D, S><<<row_grid(p), row_block(p), 0, s>>>(p, par, acc, counts);

@@ -47,25 +47,21 @@ struct Ops {
   }
   virtual void label_prep(const Params &p, cudaStream_t s) = 0;
   virtual void bubble_update(const Params &p, cudaStream_t s) = 0;
-  // a step whose added gas cells keep every bubble's cells, number and root
-  // (decided on the device after the marking, label_choose) patches the
-  // labels of the last step (label_fast) and updates one-to-one bubble
-  // groups (bubble_update_fast); the union-find kernels, the relabelling and
-  // the general bubble update return at once in such a step, the patch
-  // kernels in every other
+  // a step whose conversions keep every bubble (decided on the device by
+  // label_check after the marking): the union-find kernels return at once,
+  // label_relabel patches the labels of the last step and bubble_update
+  // updates one-to-one
   virtual void label_check(const Params &p, cudaStream_t s) = 0;  // after the marking
-  virtual void label_choose(const Params &p, cudaStream_t s) = 0;
   // at the start of the step, before the marking: label_new brought up to
-  // the last labels (see k_label_sync); label_fast then writes the patch
+  // the last labels (see k_label_sync); label_relabel then writes the patch
   virtual void label_sync(const Params &p, cudaStream_t s) = 0;
-  virtual void label_fast(const Params &p, cudaStream_t s) = 0;
-  virtual void bubble_update_fast(const Params &p, cudaStream_t s) = 0;
   virtual void geometry(const Params &p, cudaStream_t s) = 0;
   virtual void disjoining(const Params &p, cudaStream_t s) = 0;
   virtual void mlp_kappa(const Params &p, const void *img, cudaStream_t s) = 0;
   virtual void mlp_harvest(const Params &p, float *x, float *y, int *cells, int cap, int *count, cudaStream_t s) = 0;
-  // export
-  virtual void field(const Params &p, int par, int which, void *out, int dtype, cudaStream_t s) = 0;
+  // export (rank: the public numbers of the current table's slots into p.rank)
+  virtual void rank(const Params &p, cudaStream_t s) = 0;
+  virtual void fields(const Params &p, int par, unsigned mask, void *const (&out)[11], int dtype, cudaStream_t s) = 0;
   virtual void ledger(const Params &p, int par, double *acc, unsigned long long *counts, cudaStream_t s) = 0;
 };
 
