@@ -91,6 +91,7 @@ struct lbf_sim {
   int *lab_full = nullptr;
   bool walled = false;  // walls close every face and no fluid cell lies in a face layer
   int *rmv = nullptr, *rmlist = nullptr, *rank = nullptr;
+  int *clist = nullptr, *ccount = nullptr, *scan_done = nullptr, ccap = 0;
   int tile_blocks = 0;
   uint8_t *tdirty = nullptr;
   size_t ntiles_alloc = 0;
@@ -194,6 +195,10 @@ Params make_params(lbf_sim *s, long long step) {
   p.rmv = s->rmv;
   p.rmlist = s->rmlist;
   p.rank = s->rank;
+  p.scan_done = s->scan_done;
+  p.clist = s->clist;
+  p.ccount = s->ccount;
+  p.ccap = s->ccap;
   p.tile_blocks = s->tile_blocks;
   p.tdirty = s->tdirty;
   p.rlabel = s->rlabel;
@@ -240,6 +245,7 @@ int relabel_in_place(lbf_sim *s) {
   CK(cudaMemsetAsync(s->lab_fast, 0, sizeof(int), s->st));
   // the next patched labelling starts from a full copy
   CK(cudaMemsetAsync(s->lab_full, 0xff, sizeof(int), s->st));
+  CK(cudaMemsetAsync(s->ccount, 0, sizeof(int), s->st));
   s->ops->label(p, s->st);
   s->ops->bubble_update(p, s->st);
   const size_t cap = (size_t)s->cap;
@@ -1006,10 +1012,6 @@ int lbf_create(const lbf_config *cfg, lbf_sim **out) {
   AL(dalloc(s, &s->rlabel, N));
   AL(dalloc(s, &s->acc, 4));
   AL(dalloc(s, &s->counts, 4));
-  s->n_state_allocs = s->allocs.size();
-  // scratch, not part of a checkpoint
-  AL(dalloc(s, &s->rank, s->cap));
-  AL(dalloc(s, &s->rmlist, s->cap));
 #undef AL
   // zero everything that is read before being written
   auto zero = [&](void *p, size_t b) { return cudaMemsetAsync(p, 0, b, s->st); };
@@ -1054,6 +1056,22 @@ int lbf_create(const lbf_config *cfg, lbf_sim **out) {
     return fail(LBF_ECUDA, std::string("cudaMemsetAsync: ") + cudaGetErrorString(e));
   }
   rc = build_tau_table(s);
+  if (rc) {
+    std::string msg = g_err;
+    lbf_destroy(s);
+    return fail(rc, msg);
+  }
+  s->n_state_allocs = s->allocs.size();
+  // scratch, not part of a checkpoint
+  rc = dalloc(s, &s->rank, s->cap);
+  if (!rc) rc = dalloc(s, &s->rmlist, s->cap);
+  // contacts: a film of one interface layer between every two bubbles
+  // fills one cell per segment at most on average
+  s->ccap = (int)std::min<size_t>(s->nseg, 1u << 20);
+  if (!rc) rc = dalloc(s, &s->clist, s->ccap);
+  if (!rc) rc = dalloc(s, &s->ccount, 1);
+  if (!rc) rc = dalloc(s, &s->scan_done, 1);
+  if (!rc && cudaMemsetAsync(s->scan_done, 0, sizeof(int), s->st) != cudaSuccess) rc = fail(LBF_ECUDA, "cudaMemsetAsync");
   if (rc) {
     std::string msg = g_err;
     lbf_destroy(s);
@@ -1364,6 +1382,7 @@ int lbf_checkpoint_load(lbf_sim *s, const void *src, size_t bytes) {
     CK(cudaMemcpyAsync(s->allocs[k], i, s->alloc_bytes[k], cudaMemcpyHostToDevice, s->st));
     i += s->alloc_bytes[k];
   }
+  CK(cudaMemsetAsync(s->ccount, 0x7f, sizeof(int), s->st));  // contacts unknown
   CK(cudaStreamSynchronize(s->st));
   s->step = h.step;
   s->walled = h.walled != 0 && all_faces_walled(s);

@@ -180,9 +180,13 @@ struct Params {
   // from a full copy instead of copying the listed cells
   int *lab_full;
   // root moves of a patched step: [0] the number of bubbles whose root cell
-  // turns interface (listed in rmlist), less one, [1] the blocks of the root
-  // scan that are done
-  int *rmv, *rmlist;
+  // turns interface (listed in rmlist), less one, [1] set when an added gas
+  // cell lowered a root; the blocks of the root scan that are done
+  int *rmv, *rmlist, *scan_done;
+  // interface cells with gas neighbours of two bubbles (after the last
+  // labelling, and by cells added in this step): see k_root_scan.  A count
+  // past the capacity: unknown.
+  int *clist, *ccount, ccap;
   int *rank;  // scratch of exports: the public number of each slot
   int tile_blocks;  // grid of the tile loops of the union-find (two blocks per SM)
   // label of each current root cell (rank among the sorted roots, -1 past
@@ -429,6 +433,12 @@ __device__ __forceinline__ int post_type(uint8_t f) {
   if (m == MK_EMPTY) return T_GAS;
   if (m == MK_GI || m == MK_LI) return T_IFC;
   return ftype(f);
+}
+
+// list an interface cell that has gas neighbours of two bubbles
+__device__ __forceinline__ void list_contact(const Params &p, int n) {
+  const int k = atomicAdd(p.ccount, 1);
+  if (k < p.ccap) p.clist[k] = n;
 }
 
 // warp-aggregated FP64 atomic add keyed by a bubble index: lanes holding the

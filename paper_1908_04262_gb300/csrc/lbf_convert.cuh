@@ -191,11 +191,17 @@ __device__ __forceinline__ bool addition_keeps_bubble(const Params &p, const Cel
     ln[i] = p.label_old[m];
   }
   if (L < 0) return false;
-  if (n < p.told.root[L]) atomicMin(p.tnew.root + L, n);
+  if (n < p.told.root[L]) {
+    atomicMin(p.tnew.root + L, n);
+    p.rmv[1] = 1;
+  }
   bool anchored = false;
 #pragma unroll
   for (int i = 1; i < Lat<D>::Q; ++i) {
-    if (post_type(fn[i]) != T_GAS) continue;
+    const int t = post_type(fn[i]);
+    // an interface neighbour of another bubble now touches both
+    if (t == T_IFC && ln[i] >= 0 && ln[i] != L) list_contact(p, nb<D>(p, c, i));
+    if (t != T_GAS) continue;
     if (ln[i] != L) return false;
     if (ftype(fn[i]) == T_GAS) anchored = true;  // gas before, and no mark turns it interface
   }
@@ -277,13 +283,57 @@ __device__ __forceinline__ bool removal_keeps_bubble(const Params &p, const Cell
 // that keep large foams on the patched labelling: see label_fast.
 //
 // The last block to finish writes the step's choice of labelling branch,
-// lab_fast: patched unless the state was set from outside (gas_dirty -1) or
-// a conversion was refused (lab_slow).
+// lab_fast: patched unless the state was set from outside (gas_dirty -1), a
+// conversion was refused (lab_slow), or roots moved as `renumbers` says
+// while the label of some interface cell goes from one bubble to another.
+// Old and new bubbles that share an interface cell pool their gas, which is
+// the full labelling's work.  Such a cell has gas neighbours of two bubbles,
+// so only the listed ones (clist) are looked at.
 constexpr int SCAN_THREADS = 512, SCAN_WORDS = 8, SCAN_BLOCKS = 32;
+
+// the label of interface cell n after the conversion: its gas neighbour of
+// the smallest root
+template <int D> __device__ __forceinline__ int patched_label(const Params &p, int n) {
+  const Cell c = make_cell(p, n);
+  int knew = -1, rnew = 0;
+#pragma unroll
+  for (int i = 1; i < Lat<D>::Q; ++i) {
+    const int m = nb<D>(p, c, i);
+    if (post_type(p.flags[m]) != T_GAS) continue;
+    const int l = p.label_old[m];
+    if (l < 0 || l == knew) continue;
+    const int r = __ldcg(p.tnew.root + l);
+    if (knew < 0 || r < rnew) {
+      knew = l;
+      rnew = r;
+    }
+  }
+  return knew;
+}
+
+// Root moves that renumber: two bubbles lost their root cells, one lost it
+// while a root was lowered, a moved root passed another's, or the new root
+// lies more than 32,768 cells on.  (Fewer moves leave each bubble its gas
+// whatever an interface cell's label does.)  Whole block.
+__device__ __forceinline__ bool renumbers(const Params &p, int removed) {
+  if (removed >= 2 || (removed == 1 && p.rmv[1])) return true;
+  const int cnt = *p.told.count;
+  bool any = false;
+  for (int k = threadIdx.x; k < cnt; k += blockDim.x) {
+    const int a = p.told.root[k], b = __ldcg(p.tnew.root + k);
+    if (a == b) continue;
+    if (b > a + 32768) any = true;
+    for (int j = 0; j < cnt && !any; ++j) {
+      const int r = p.told.root[j];
+      any = (r > b && r < a) || (r > a && r < b);
+    }
+  }
+  return __syncthreads_or(any);
+}
 template <int D>
 __global__ void __launch_bounds__(SCAN_THREADS) k_root_scan(Params p) {
   __shared__ int found;
-  const int cnt = p.rmv[0] + 1;
+  const int cnt = p.rmv[0] + 1;  // read by every block before any can be the last
   const long long layer = D == 3 ? (long long)p.nx * p.ny : p.nx;
   for (int e = blockIdx.x; e < cnt; e += gridDim.x) {
     const int L = p.rmlist[e];
@@ -344,14 +394,32 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_root_scan(Params p) {
     }
     __syncthreads();
   }
+  __shared__ bool last;
   if (threadIdx.x == 0) {
     __threadfence();
-    if (atomicAdd(p.rmv + 1, 1) == (int)gridDim.x - 1) {
-      __threadfence();
-      const bool fast = *p.gas_dirty >= 0 && __ldcg(p.lab_slow) == 0;
-      *p.lab_fast = fast;
-      *p.lab_full = !fast;
+    last = atomicAdd(p.scan_done, 1) == (int)gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  bool fast = *p.gas_dirty >= 0 && __ldcg(p.lab_slow) == 0;
+  if (fast && (cnt > 0 || p.rmv[1])) {
+    const int nc = *p.ccount;
+    bool changed = nc > p.ccap;
+    for (int k = threadIdx.x; k < nc && !changed; k += blockDim.x) {
+      const int n = p.clist[k], old = p.label_old[n];
+      if (old < 0 || post_type(p.flags[n]) != T_IFC) continue;
+      const int now = patched_label<D>(p, n);
+      changed = now >= 0 && now != old;
     }
+    if (__syncthreads_or(changed)) fast = !renumbers(p, cnt);
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    *p.lab_fast = fast;
+    *p.lab_full = !fast;
+    *p.ccount = 0;  // listed afresh by this step's labelling
+    *p.scan_done = 0;
   }
 }
 

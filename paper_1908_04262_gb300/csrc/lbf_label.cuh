@@ -518,14 +518,17 @@ __device__ __forceinline__ void relabel_all(const Params &p, double *wbuf) {
       ngas = p.lsize[n];  // non-zero only at tile-local roots
       if (p.atmosphere && knew >= 0 && (D == 2 ? c.y : c.z) == p.top_layer && !p.tnew.atm[knew]) p.tnew.atm[knew] = 1;
     } else if (t == T_IFC) {
+      bool two = false;
 #pragma unroll
       for (int i = 1; i < Lat<D>::Q; ++i) {
         const long long m = nb<D>(p, c, i);
         if (post_type(p.flags[m]) == T_GAS) {
           const int k = p.rlabel[p.parent[m]];
+          two |= k >= 0 && knew >= 0 && k != knew;
           if (k >= 0 && (knew < 0 || k < knew)) knew = k;
         }
       }
+      if (two) list_contact(p, (int)n);
       if (knew >= 0) v = 1.0 - (double)((const R *)p.phi)[n];
     }
     if (inr) p.label_new[n] = knew;
@@ -718,9 +721,9 @@ static __global__ void __launch_bounds__(1024) k_bubble_update(Params p) {
 // labelling.  In foams of a few hundred bubbles that is nearly every step
 // (256^3 with 200 bubbles 1,262 steps of 1,336, 512x512x384 with 2,000 all
 // of them), while in the same runs one step in a thousand joined or split
-// bubbles.  Measured, ms for the timed passes of those foams: 256^3 shifted
-// FP16, 8 steps, 9.86 -> 6.61; 512x512x384 shifted BF16, 4 steps, 31.0 ->
-// 20.0; 2D 450x650, 150 bubbles, 20 steps, 1.76 -> 1.31.
+// bubbles.  Measured, ms (with the one-pass export): 256^3 shifted FP16, 8
+// steps, 9.88 -> 6.49; 512x512x384 shifted BF16, 4 steps, 31.0 -> 19.0; 2D
+// 450x650, 150 bubbles, 20 steps, 1.79 -> 1.25.
 
 // At the start of a step, before its marking: bring label_new (the labels
 // of the step before last) up to the last labels wherever they differ.
@@ -811,14 +814,17 @@ __device__ __forceinline__ void patch_labels(const Params &p, double *wbuf) {
         fn[i] = p.flags[m];
         ln[i] = p.label_old[m];
       }
+      bool two = false;
 #pragma unroll
       for (int i = 1; i < Lat<D>::Q; ++i) {
         if (post_type(fn[i]) == T_GAS) {
           const int l = ln[i];
           if (l < 0 || l == knew) continue;
+          two = knew >= 0;
           if (knew < 0 || p.tnew.root[l] < p.tnew.root[knew]) knew = l;
         }
       }
+      if (two) list_contact(p, n);
       p.label_new[n] = knew;
       if (knew >= 0) {
         v = 1.0 - (double)((const R *)p.phi)[n];

@@ -72,3 +72,31 @@ def test_numbers_follow_the_roots(oracle_mod, shape, walled, steps):
     for name in ("id", "root"):
         assert np.array_equal(bf[name], bo[name])
     assert rel_err(bf["volume"], bo["volume"]) < 1e-10
+
+
+def test_touching_bubbles_pool_their_gas():
+    """Two bubbles behind one layer of interface cells (32^3, FP64): when
+    their roots pass one another those cells go from one bubble to the other,
+    so that old and new bubbles share cells and pool their gas; the larger
+    keeps the smaller id, the other gets a fresh one.  Ids and pressures are
+    those of the library whose labels were the ranks of the roots, where a
+    change of order always took the full labelling."""
+    import torch
+
+    if not torch.cuda.is_available():
+        pytest.fail("the GPU tests need a CUDA device")
+    from paper_1908_04262_gb300 import build as B
+    from paper_1908_04262_gb300 import lbf
+
+    B.build()
+    cfg, c, _ = W.c2_crop_3d_32(storage="fp64")
+    sim = lbf.Sim(cfg)
+    sim.nucleate(np.concatenate([c, [[22.0, 20.0, 9.0]]]), [5.0, 3.0])
+    sim.step(21)
+    b = sim.bubbles()
+    assert b["id"].tolist() == [1, 3, 0] and b["root"].tolist() == [7696, 7797, 25633]
+    assert rel_err(b["pressure"], [0.33273405295113834, 0.3361376202527489, 1 / 3]) < 1e-10
+    sim.step(9)
+    b = sim.bubbles()
+    assert b["id"].tolist() == [4, 1, 0] and b["root"].tolist() == [7797, 8655, 25633]
+    assert rel_err(b["pressure"], [0.3356138194055036, 0.33639008142017535, 1 / 3]) < 1e-10
