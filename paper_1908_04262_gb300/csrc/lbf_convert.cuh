@@ -296,12 +296,18 @@ constexpr int SCAN_THREADS = 512, SCAN_WORDS = 8, SCAN_BLOCKS = 32;
 template <int D> __device__ __forceinline__ int patched_label(const Params &p, int n) {
   const Cell c = make_cell(p, n);
   int knew = -1, rnew = 0;
+  uint8_t fn[Lat<D>::Q];
+  int ln[Lat<D>::Q];
 #pragma unroll
   for (int i = 1; i < Lat<D>::Q; ++i) {
     const int m = nb<D>(p, c, i);
-    if (post_type(p.flags[m]) != T_GAS) continue;
-    const int l = p.label_old[m];
-    if (l < 0 || l == knew) continue;
+    fn[i] = p.flags[m];
+    ln[i] = p.label_old[m];
+  }
+#pragma unroll
+  for (int i = 1; i < Lat<D>::Q; ++i) {
+    const int l = ln[i];
+    if (post_type(fn[i]) != T_GAS || l < 0 || l == knew) continue;
     const int r = __ldcg(p.tnew.root + l);
     if (knew < 0 || r < rnew) {
       knew = l;

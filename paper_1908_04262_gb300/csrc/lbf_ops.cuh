@@ -51,11 +51,19 @@ struct OpsImpl final : Ops {
     k_nucleate<D, S><<<blocks_for(cnt, B), B, 0, s>>>(p, par, c[0], c[1], D == 3 ? c[2] : 0.0, R0, x0, y0,
                                                         z0, bx, by, bz);
   }
+  // more segments than the grid has warps (four a block)
+  static bool packs(const Params &p, int blocks) {
+    return (long long)((p.nx + 31) / 32) * p.ny * p.nz > 4ll * blocks;
+  }
+  template <bool WALLED, bool PACK> void exchange_as(const Params &p, int par, cudaStream_t s) {
+    par ? k_exchange<D, S, 1, WALLED, PACK><<<p.warp_blocks, 128, 0, s>>>(p)
+        : k_exchange<D, S, 0, WALLED, PACK><<<p.warp_blocks, 128, 0, s>>>(p);
+  }
   void exchange(const Params &p, int par, cudaStream_t s) override {
-    if (p.walled)
-      par ? k_exchange<D, S, 1, true><<<p.warp_blocks, 128, 0, s>>>(p) : k_exchange<D, S, 0, true><<<p.warp_blocks, 128, 0, s>>>(p);
+    if (packs(p, p.warp_blocks))
+      p.walled ? exchange_as<true, true>(p, par, s) : exchange_as<false, true>(p, par, s);
     else
-      par ? k_exchange<D, S, 1><<<p.warp_blocks, 128, 0, s>>>(p) : k_exchange<D, S, 0><<<p.warp_blocks, 128, 0, s>>>(p);
+      p.walled ? exchange_as<true, false>(p, par, s) : exchange_as<false, false>(p, par, s);
   }
   void build_ilist(const Params &p, cudaStream_t s) override {
     cudaMemsetAsync(p.icount, 0, sizeof(int), s);
@@ -77,18 +85,24 @@ struct OpsImpl final : Ops {
     else
       par ? k_stream_liquid<D, S, 1, 0><<<g, b, 0, s>>>(p) : k_stream_liquid<D, S, 0, 0><<<g, b, 0, s>>>(p);
   }
-  void stream_interface(const Params &p, int par, cudaStream_t s) override {
+  template <int COLL, bool WALLED> void interface_as(const Params &p, int par, cudaStream_t s) {
     const int g = p.list_blocks;
-    if (p.coll == 2)
-      par ? k_stream_interface<D, S, 1, 2><<<g, 128, 0, s>>>(p) : k_stream_interface<D, S, 0, 2><<<g, 128, 0, s>>>(p);
-    else if (p.coll == 1)
-      par ? k_stream_interface<D, S, 1, 1><<<g, 128, 0, s>>>(p) : k_stream_interface<D, S, 0, 1><<<g, 128, 0, s>>>(p);
-    else if (p.walled)
-      par ? k_stream_interface<D, S, 1, 0, true><<<g, 128, 0, s>>>(p)
-          : k_stream_interface<D, S, 0, 0, true><<<g, 128, 0, s>>>(p);
+    if (packs(p, g))
+      par ? k_stream_interface<D, S, 1, COLL, WALLED, true><<<g, 128, 0, s>>>(p)
+          : k_stream_interface<D, S, 0, COLL, WALLED, true><<<g, 128, 0, s>>>(p);
     else
-      par ? k_stream_interface<D, S, 1, 0><<<g, 128, 0, s>>>(p)
-          : k_stream_interface<D, S, 0, 0><<<g, 128, 0, s>>>(p);
+      par ? k_stream_interface<D, S, 1, COLL, WALLED, false><<<g, 128, 0, s>>>(p)
+          : k_stream_interface<D, S, 0, COLL, WALLED, false><<<g, 128, 0, s>>>(p);
+  }
+  void stream_interface(const Params &p, int par, cudaStream_t s) override {
+    if (p.coll == 2)
+      interface_as<2, false>(p, par, s);
+    else if (p.coll == 1)
+      interface_as<1, false>(p, par, s);
+    else if (p.walled)
+      interface_as<0, true>(p, par, s);
+    else
+      interface_as<0, false>(p, par, s);
   }
   void convert_mark(const Params &p, cudaStream_t s) override { k_conv_mark<D><<<p.list_blocks, 128, 0, s>>>(p); }
   void convert_excess(const Params &p, int par, cudaStream_t s) override {

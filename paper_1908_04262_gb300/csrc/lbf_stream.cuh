@@ -112,28 +112,26 @@ template <class R> __device__ __forceinline__ R solve_tau(const Params &p, R A) 
   return t;
 }
 
-// one warp per segment of interface cells, one lane per cell (loads along x
-// coalesce like the lattice sweep's)
-template <int D, class S, int PAR, bool WALLED = false>
+// the cells of the segment list, one lane each (neighbours along x coalesce
+// like the lattice sweep's)
+template <int D, class S, int PAR, bool WALLED, bool PACK>
 __global__ void __launch_bounds__(128) k_exchange(Params p) {
   using R = typename ST<S>::R;
   constexpr int Q = Lat<D>::Q;
-  const int lane = threadIdx.x & 31;
-  const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int nwarps = (gridDim.x * blockDim.x) >> 5;
+  __shared__ unsigned s_mask[128], s_first[128];
   const int cnt = *p.segcount;
   const S *f = (const S *)p.f;
   R *M = (R *)p.M;
   const R *phi = (const R *)p.phi;
   // the step's first kernel: the interface sweep lists marked cells afresh
   if (blockIdx.x == 0 && threadIdx.x == 0) *p.mcount = 0;
-  for (int k = warp; k < cnt; k += nwarps) {
-    Cell c;
-    if (!(WALLED ? seg_cell_walled(p, p.seglist[k], lane, c) : seg_cell(p, p.seglist[k], lane, c))) continue;
+  const int wb = threadIdx.x & ~31;
+  // types through the last conversion's marks: the exchange may run while
+  // that conversion still writes the new types
+  auto take = [](uint8_t fl) { return post_type(fl) == T_IFC; };
+  for_segment_cells<WALLED, PACK>(p, p.seglist, cnt, s_mask + wb, s_first + wb, take, [&](const Cell &c, bool on) {
+    if (!on) return;
     const int n = c.n;
-    // types through the last conversion's marks: the exchange may run while
-    // that conversion still writes the new types
-    if (post_type(p.flags[n]) != T_IFC) continue;
     const R phn = phi[n];
     // every load issued at once (none waits for a neighbour's type; the
     // slots and fill levels of gas and wall neighbours are read and unused)
@@ -169,7 +167,7 @@ __global__ void __launch_bounds__(128) k_exchange(Params p) {
     uI[p.N + n] = (jy - (R)0.5 * rho * PV(R, ay)) * irho;
     uI[2 * p.N + n] = (jz - (R)0.5 * rho * PV(R, az)) * irho;
     M[n] = M[n] + dM;
-  }
+  });
 }
 
 template <class R> struct SweepOcc;
@@ -661,34 +659,30 @@ __device__ __forceinline__ int interface_cell(const Params &p, const Cell &c, lo
   return mk;
 }
 
-// the interface cells of the step, one warp per segment of the segment list
-// and one lane per cell; cells that fill or empty are listed for the
-// conversion.  Block 0 also resets the counters of the lists that the
-// conversion fills.
-template <int D, class S, int PAR, int COLL, bool WALLED = false>
+// the interface cells of the step, one lane each (for_segment_cells); cells
+// that fill or empty are listed for the conversion.  Block 0 also resets the
+// counters of the lists that the conversion fills.
+template <int D, class S, int PAR, int COLL, bool WALLED, bool PACK>
 __global__ void __launch_bounds__(128, 4) k_stream_interface(Params p) {
   __shared__ double wbuf[128];
-  const int lane = threadIdx.x & 31;
-  const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int nwarps = (gridDim.x * blockDim.x) >> 5;
+  __shared__ unsigned s_mask[128], s_first[128];
   const int cnt = *p.segcount;
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     *p.ncount = 0;
     *p.segnext_count = 0;
     if (p.pf.q != 0.f) atomicAdd(p.fluid_updates, (unsigned long long)*p.icount);
   }
-  for (int k = warp; k < cnt; k += nwarps) {
-    const int seg = p.seglist[k];
-    Cell c;
-    const bool inr = WALLED ? seg_cell_walled(p, seg, lane, c) : seg_cell(p, seg, lane, c);
-    const uint8_t fl = inr ? p.flags[c.n] : (uint8_t)T_GAS;
+  // the segments' list flags: free for the conversion's next list
+  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < cnt; k += gridDim.x * blockDim.x) p.segflag[p.seglist[k]] = 0;
+  const int wb = threadIdx.x & ~31;
+  auto take = [](uint8_t fl) { return ftype(fl) == T_IFC; };
+  for_segment_cells<WALLED, PACK>(p, p.seglist, cnt, s_mask + wb, s_first + wb, take, [&](const Cell &c, bool on) {
     double flux = 0.0;
     int lab = -1, mk = MK_NONE;
-    if (ftype(fl) == T_IFC) mk = interface_cell<D, S, PAR, COLL>(p, c, c.n, fl, flux, lab);
-    if (lane == 0) p.segflag[seg] = 0;  // free for the conversion's next list
+    if (on) mk = interface_cell<D, S, PAR, COLL>(p, c, c.n, p.flags[c.n], flux, lab);
     list_append(p.mlist, p.mcount, mk != MK_NONE, c.n);
-    if (__any_sync(0xffffffffu, lab >= 0)) agg_add(p.told.dm, lab, flux, wbuf + (threadIdx.x & ~31));
-  }
+    if (__any_sync(0xffffffffu, lab >= 0)) agg_add(p.told.dm, lab, flux, wbuf + wb);
+  });
 }
 
 }  // namespace lbf
