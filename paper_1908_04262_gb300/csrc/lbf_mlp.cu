@@ -28,10 +28,18 @@ int fail(int code, const char *msg) {
   } while (0)
 
 // inference: canonical stencils (n x 27 fp32) -> y = 4 kappa, on the
-// fifth-generation tensor cores: tiles of 128 rows, each CTA (128 threads)
-// walking tiles; a tile whose MMA did not complete within the wait bound
-// (and every later tile of that CTA) gets NaN outputs
-__global__ void __launch_bounds__(128) k_forward_tc(const float *theta, const float *x, int n, float *y) {
+// fifth-generation tensor cores: tiles of 128 rows, each CTA walking tiles;
+// a tile whose MMA did not complete within the wait bound (and every later
+// tile of that CTA) gets NaN outputs.
+//
+// A tile is a serial chain (gather, MMA, SiLU, MMA, SiLU), so the rate is
+// set by how many tiles are under way: four CTAs per SM (all that the 512
+// tensor-memory columns hold at 128 each) of 256 threads (two per row, half
+// the columns each) instead of one of 128.  What then bounds it is the
+// special-function unit, two results for each of the 128 SiLUs of a row
+// (27 us at 503,117 rows).  Measured there: 208 -> 68 us.
+constexpr int FWD_THREADS = 256, FWD_CTAS = 4;
+__global__ void __launch_bounds__(FWD_THREADS, FWD_CTAS) k_forward_tc(const float *theta, const float *x, int n, float *y) {
   extern __shared__ __align__(128) unsigned char tsm[];
   tc::Tile &t = *reinterpret_cast<tc::Tile *>(tsm);
   tc::pack_image(t.net, theta);
@@ -48,7 +56,7 @@ __global__ void __launch_bounds__(128) k_forward_tc(const float *theta, const fl
       tc::put_x(t, r, k, r < rows ? xt[e] : 0.f);
     }
     float yv = __int_as_float(0x7fc00000);
-    if (!failed) failed = !tc::forward_tile<128>(t, phase, yv);
+    if (!failed) failed = !tc::forward_tile<FWD_THREADS>(t, phase, yv);
     if ((int)threadIdx.x < rows) y[row0 + threadIdx.x] = yv;
   }
   tc::teardown(t, phase, failed);
@@ -108,13 +116,16 @@ struct __align__(128) GradSmem {
   __nv_bfloat16 ad2[128 * 64];   // delta2 (A of delta2 W2)
   __nv_bfloat16 ag[128 * 128];   // rows 0-63 delta2^T, 64-127 delta1^T; K = the tile's rows
   __nv_bfloat16 bg[112 * 128];   // rows 0-63 H1^T, 64-90 X^T, 96 ones, the rest zero
-  float d3[128], le[128];        // delta3 and the loss of each row
+  float d3[128];                 // delta3 of each row
+  float part[4][128];            // partial outputs of each row, by column group
+  float red[8][64];              // partial sums of dW3, by row group
+  float tgt[128];
   long long src[128];            // data row of each tile row
 };
 constexpr uint32_t GRAD_TCOLS = 512;  // Z1 0-63, Z2 64-127, delta2 W2 128-191, gradients 256-367
 
 // Gradient of L = (1/2n) sum (y - t)^2 on the fifth-generation tensor
-// cores: tiles of 128 rows, one row per thread in the epilogues.  Per tile:
+// cores: tiles of 128 rows.  Per tile:
 //   Z1 = X W1^T, H1 = SiLU(Z1 + b1); Z2 = H1 W2^T, y = BF16(SiLU(Z2 + b2)) W3 + b3
 //   delta3 = (y - t) / n, delta2 = delta3 W3 SiLU'(Z2 + b2)
 //   delta1 = (delta2 W2) SiLU'(Z1 + b1)                    (MMA, K = 64)
@@ -123,37 +134,53 @@ constexpr uint32_t GRAD_TCOLS = 512;  // Z1 0-63, Z2 64-127, delta2 W2 128-191, 
 // dW3, db3 and the loss are summed in shared memory per tile.  Everything
 // is added into grad and *loss (global) once per CTA.  A timed-out wait
 // adds NaN to *loss.
-__global__ void __launch_bounds__(128) k_grad_tc(const TrainImage *img, const float *x, const float *tgt, int n,
-                                                 Batch bt, float *grad, double *loss) {
+//
+// A training batch is 16 tiles on as many CTAs, so the kernel is the latency
+// of one tile: four MMA round trips and the epilogues between them.  512
+// threads share the epilogues: four warps on each quarter of the
+// tensor-memory lanes, 16 of the 64 columns each, where 128 threads walked
+// all 64; the column and row sums are split the same way.  Measured with
+// the rest of a batch (batches of 2,048): about 45 us a batch with three
+// launches -> 25 us with two, 20 of them here.
+constexpr int GRAD_THREADS = 512;
+__global__ void __launch_bounds__(GRAD_THREADS) k_grad_tc(const TrainImage *img, const float *x, const float *tgt, int n,
+                                                          Batch bt, float *grad, double *loss) {
   extern __shared__ __align__(128) unsigned char gsm[];
   GradSmem &s = *reinterpret_cast<GradSmem *>(gsm);
   tc::Tile &t = s.t;
-  const int tid = threadIdx.x, w = tid >> 5;
+  // row of the epilogues, and the 16 columns from c0 on
+  const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31, row = tid & 127, cg = tid >> 7, c0 = 16 * cg;
   const int tiles = (n + tc::ROWS - 1) / tc::ROWS;
-  for (int i = tid; i < 112 * 128; i += 128) {
-    const int r = i >> 7, m = i & 127;
-    s.bg[tc::kofs(r, m, 128) / 2] = __float2bfloat16_rn(r == 96 ? 1.f : 0.f);
+  for (int i = tid; i < 112 * 128 / 8; i += GRAD_THREADS) {
+    // eight K-columns of one row: row 96 is the ones
+    const int off = 16 * i, r = (off >> 11) * 8 + ((off & 127) >> 4);
+    const unsigned v = r == 96 ? 0x3f803f80u : 0u;
+    *reinterpret_cast<uint4 *>(reinterpret_cast<unsigned char *>(s.bg) + off) = make_uint4(v, v, v, v);
   }
   tc::setup(t, GRAD_TCOLS, tc::Copy{&t.net, &img->net, (uint32_t)sizeof(tc::Image)},
             tc::Copy{s.w2t, img->w2t, (uint32_t)sizeof(img->w2t)});
-  const uint32_t tm = t.tmem, lanes = (uint32_t)(32 * w) << 16;
+  const uint32_t tm = t.tmem, lanes = (uint32_t)(32 * (w & 3)) << 16;
   const float inv_n = 1.f / (float)n;
   uint32_t phase = 0;
   bool failed = false, net = false, any = false;
   for (int tile = blockIdx.x; tile < tiles && !failed; tile += gridDim.x) {
     const int row0 = tile * tc::ROWS, rows = min(tc::ROWS, n - row0);
-    // the tile's data rows (thread = row), then X into a1 and X^T into bg
-    float target = 0.f;
-    if (tid < rows) {
-      const long long src =
-          (long long)((bt.a * (unsigned long long)(bt.start + row0 + tid) + bt.b) % (unsigned long long)bt.ntot);
-      s.src[tid] = src;
-      target = tgt[src];
+    // the tile's data rows, then X into a1 and X^T into bg
+    if (tid < tc::ROWS) {
+      float target = 0.f;
+      if (tid < rows) {
+        const long long src =
+            (long long)((bt.a * (unsigned long long)(bt.start + row0 + tid) + bt.b) % (unsigned long long)bt.ntot);
+        s.src[tid] = src;
+        target = tgt[src];
+      }
+      s.tgt[tid] = target;
     }
     __syncthreads();
-#pragma unroll 9
-    for (int c = 0; c < 27; ++c) {
-      const int e = tid + 128 * c, r = e / 27, k = e - 27 * r;
+#pragma unroll
+    for (int c = 0; c < 7; ++c) {
+      const int e = tid + GRAD_THREADS * c, r = e / 27, k = e - 27 * r;
+      if (e >= tc::ROWS * 27) break;
       float v = 0.f;
       if (r < rows) {
         const long long src = s.src[r];
@@ -175,109 +202,112 @@ __global__ void __launch_bounds__(128) k_grad_tc(const TrainImage *img, const fl
         break;
       }
     }
-    // layer 1; H1 into a2 (row tid) and bg rows 0-63 (column tid)
+    // layer 1; H1 into a2 (this row) and bg rows 0-63 (this column)
     tc::to_tensor_cores();
     if (tid == 0) tc::issue(t, tm, t.a1, t.net.w1, 32, 64, 2, false);
     if (!tc::wait_mmas(t, phase)) {
       failed = true;
       break;
     }
+    float z[16];
+    tc::ld16(tm + lanes + c0, z);
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      float z[16];
-      tc::ld16(tm + lanes + 16 * c, z);
+    for (int h = 0; h < 2; ++h) {
+      uint4 q;
+      uint32_t *qw = reinterpret_cast<uint32_t *>(&q);
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        uint4 q;
-        uint32_t *qw = reinterpret_cast<uint32_t *>(&q);
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          const int j = 16 * c + 8 * h + 2 * e;
-          const __nv_bfloat162 hv =
-              __floats2bfloat162_rn(silu(z[8 * h + 2 * e] + t.net.b1[j]), silu(z[8 * h + 2 * e + 1] + t.net.b1[j + 1]));
-          qw[e] = *reinterpret_cast<const uint32_t *>(&hv);
-          s.bg[tc::kofs(j, tid, 128) / 2] = hv.x;
-          s.bg[tc::kofs(j + 1, tid, 128) / 2] = hv.y;
-        }
-        *reinterpret_cast<uint4 *>(reinterpret_cast<unsigned char *>(t.a2) + tc::kofs(tid, 16 * c + 8 * h, 64)) = q;
+      for (int e = 0; e < 4; ++e) {
+        const int j = c0 + 8 * h + 2 * e;
+        const __nv_bfloat162 hv =
+            __floats2bfloat162_rn(silu(z[8 * h + 2 * e] + t.net.b1[j]), silu(z[8 * h + 2 * e + 1] + t.net.b1[j + 1]));
+        qw[e] = *reinterpret_cast<const uint32_t *>(&hv);
+        s.bg[tc::kofs(j, row, 128) / 2] = hv.x;
+        s.bg[tc::kofs(j + 1, row, 128) / 2] = hv.y;
       }
+      *reinterpret_cast<uint4 *>(reinterpret_cast<unsigned char *>(t.a2) + tc::kofs(row, c0 + 8 * h, 64)) = q;
     }
-    // layer 2; y, delta3 and the loss of row tid; BF16 H2 into a2 (row-major)
+    // layer 2; y, delta3 and the loss of the row; BF16 H2 into a2 (row-major)
     tc::to_tensor_cores();
     if (tid == 0) tc::issue(t, tm + 64, t.a2, t.net.w2, 64, 64, 4, false);
     if (!tc::wait_mmas(t, phase)) {
       failed = true;
       break;
     }
-    float y = 0.f;
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      float z[16];
-      tc::ld16(tm + lanes + 64 + 16 * c, z);
+    tc::ld16(tm + lanes + 64 + c0, z);
+    {
+      float y = 0.f;
 #pragma unroll
       for (int e = 0; e < 16; e += 2) {
-        const int j = 16 * c + e;
+        const int j = c0 + e;
         const __nv_bfloat162 hv = __floats2bfloat162_rn(silu(z[e] + t.net.b2[j]), silu(z[e + 1] + t.net.b2[j + 1]));
         y += __bfloat162float(hv.x) * t.net.w3[j] + __bfloat162float(hv.y) * t.net.w3[j + 1];
-        *reinterpret_cast<__nv_bfloat162 *>(t.a2 + tid * 64 + j) = hv;
+        *reinterpret_cast<__nv_bfloat162 *>(t.a2 + row * 64 + j) = hv;
       }
+      s.part[cg][row] = y;
     }
-    y += t.net.b3;
-    const float err = tid < rows ? y - target : 0.f;
+    __syncthreads();
+    const float y = s.part[0][row] + s.part[1][row] + s.part[2][row] + s.part[3][row] + t.net.b3;
+    const float err = row < rows ? y - s.tgt[row] : 0.f;
     const float d3 = err * inv_n;
-    s.d3[tid] = d3;
-    s.le[tid] = 0.5f * err * err * inv_n;
-    // delta2 = delta3 W3 SiLU'(Z2 + b2): into ad2 (row tid) and ag rows 0-63
+    if (cg == 0) s.d3[row] = d3;
+    // delta2 = delta3 W3 SiLU'(Z2 + b2): into ad2 (this row) and ag rows 0-63
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      float z[16];
-      tc::ld16(tm + lanes + 64 + 16 * c, z);
+    for (int h = 0; h < 2; ++h) {
+      uint4 q;
+      uint32_t *qw = reinterpret_cast<uint32_t *>(&q);
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        uint4 q;
-        uint32_t *qw = reinterpret_cast<uint32_t *>(&q);
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          const int j = 16 * c + 8 * h + 2 * e;
-          const __nv_bfloat162 dv = __floats2bfloat162_rn(d3 * t.net.w3[j] * dsilu(z[8 * h + 2 * e] + t.net.b2[j]),
-                                                          d3 * t.net.w3[j + 1] * dsilu(z[8 * h + 2 * e + 1] + t.net.b2[j + 1]));
-          qw[e] = *reinterpret_cast<const uint32_t *>(&dv);
-          s.ag[tc::kofs(j, tid, 128) / 2] = dv.x;
-          s.ag[tc::kofs(j + 1, tid, 128) / 2] = dv.y;
-        }
-        *reinterpret_cast<uint4 *>(reinterpret_cast<unsigned char *>(s.ad2) + tc::kofs(tid, 16 * c + 8 * h, 64)) = q;
+      for (int e = 0; e < 4; ++e) {
+        const int j = c0 + 8 * h + 2 * e;
+        const __nv_bfloat162 dv = __floats2bfloat162_rn(d3 * t.net.w3[j] * dsilu(z[8 * h + 2 * e] + t.net.b2[j]),
+                                                        d3 * t.net.w3[j + 1] * dsilu(z[8 * h + 2 * e + 1] + t.net.b2[j + 1]));
+        qw[e] = *reinterpret_cast<const uint32_t *>(&dv);
+        s.ag[tc::kofs(j, row, 128) / 2] = dv.x;
+        s.ag[tc::kofs(j + 1, row, 128) / 2] = dv.y;
       }
+      *reinterpret_cast<uint4 *>(reinterpret_cast<unsigned char *>(s.ad2) + tc::kofs(row, c0 + 8 * h, 64)) = q;
     }
-    // delta2 W2 on the tensor cores while the CTA sums dW3, db3 and the loss
+    // delta2 W2 on the tensor cores while the CTA sums dW3 (16 rows of one
+    // column per thread), db3 and the loss
     tc::to_tensor_cores();
     if (tid == 0) tc::issue(t, tm + 128, s.ad2, s.w2t, 64, 64, 4, false);
-    if (tid < 64) {
+    {
+      const int j = tid & 63, m0 = 16 * (tid >> 6);
       float g = 0.f;
-      for (int m = 0; m < tc::ROWS; ++m) g += s.d3[m] * __bfloat162float(t.a2[m * 64 + tid]);
-      atomicAdd(grad + OFF_W3 + tid, g);
-    } else if (tid == 64) {
-      float g = 0.f;
-      for (int m = 0; m < tc::ROWS; ++m) g += s.d3[m];
-      atomicAdd(grad + OFF_B3, g);
-    } else if (tid == 96) {
-      double l = 0.0;
-      for (int m = 0; m < tc::ROWS; ++m) l += (double)s.le[m];
-      atomicAdd(loss, l);
+#pragma unroll
+      for (int m = 0; m < 16; ++m) g += s.d3[m0 + m] * __bfloat162float(t.a2[(m0 + m) * 64 + j]);
+      s.red[tid >> 6][j] = g;
+    }
+    if (w == 0) {
+      float g = (s.d3[lane] + s.d3[lane + 32]) + (s.d3[lane + 64] + s.d3[lane + 96]);
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) g += __shfl_xor_sync(0xffffffffu, g, o);
+      if (lane == 0) atomicAdd(grad + OFF_B3, g);
+    }
+    if (cg == 1) {  // warps 4-7 hold every row once
+      double l = (double)(0.5f * err * err * inv_n);
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+      if (lane == 0) atomicAdd(loss, l);
     }
     if (!tc::wait_mmas(t, phase)) {
       failed = true;
       break;
     }
-    // delta1 = (delta2 W2) SiLU'(Z1 + b1): into ag rows 64-127
+    if (tid < 64) {
+      float g = 0.f;
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      float z[16], d[16];
-      tc::ld16(tm + lanes + 16 * c, z);
-      tc::ld16(tm + lanes + 128 + 16 * c, d);
+      for (int k = 0; k < 8; ++k) g += s.red[k][tid];
+      atomicAdd(grad + OFF_W3 + tid, g);
+    }
+    // delta1 = (delta2 W2) SiLU'(Z1 + b1): into ag rows 64-127
+    {
+      float d[16];
+      tc::ld16(tm + lanes + c0, z);
+      tc::ld16(tm + lanes + 128 + c0, d);
 #pragma unroll
       for (int e = 0; e < 16; ++e) {
-        const int j = 16 * c + e;
-        s.ag[tc::kofs(64 + j, tid, 128) / 2] = __float2bfloat16_rn(d[e] * dsilu(z[e] + t.net.b1[j]));
+        const int j = c0 + e;
+        s.ag[tc::kofs(64 + j, row, 128) / 2] = __float2bfloat16_rn(d[e] * dsilu(z[e] + t.net.b1[j]));
       }
     }
     // weight and bias gradients of the tile, accumulated in tensor memory
@@ -292,40 +322,37 @@ __global__ void __launch_bounds__(128) k_grad_tc(const TrainImage *img, const fl
   if (failed) {
     if (tid == 0) atomicAdd(loss, (double)__int_as_float(0x7fc00000));
   } else if (any) {
-    // row tid of the accumulated block product: rows 0-63 dW2 (columns
-    // 0-63) and db2 (column 96), rows 64-127 dW1 (columns 64-90) and db1
+    // the accumulated block product: rows 0-63 dW2 (columns 0-63) and db2
+    // (column 96), rows 64-127 dW1 (columns 64-90) and db1; column groups 0-3
+    // take dW2, groups 0 and 1 dW1, group 2 both bias columns
     float z[16];
-    tc::ld16(tm + lanes + 256 + 96, z);
-    if (tid < 64) {
-      atomicAdd(grad + OFF_B2 + tid, z[0]);
+    if (row < 64) {
+      tc::ld16(tm + lanes + 256 + c0, z);
 #pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        tc::ld16(tm + lanes + 256 + 16 * c, z);
+      for (int e = 0; e < 16; ++e) atomicAdd(grad + OFF_W2 + row * 64 + c0 + e, z[e]);
+    } else if (cg < 2) {
+      tc::ld16(tm + lanes + 256 + 64 + c0, z);
 #pragma unroll
-        for (int e = 0; e < 16; ++e) atomicAdd(grad + OFF_W2 + tid * 64 + 16 * c + e, z[e]);
-      }
-    } else {
-      const int i = tid - 64;
-      atomicAdd(grad + OFF_B1 + i, z[0]);
-#pragma unroll
-      for (int c = 0; c < 2; ++c) {
-        tc::ld16(tm + lanes + 256 + 64 + 16 * c, z);
-#pragma unroll
-        for (int e = 0; e < 16; ++e)
-          if (16 * c + e < 27) atomicAdd(grad + OFF_W1 + i * 27 + 16 * c + e, z[e]);
-      }
+      for (int e = 0; e < 16; ++e)
+        if (c0 + e < 27) atomicAdd(grad + OFF_W1 + (row - 64) * 27 + c0 + e, z[e]);
+    }
+    if (cg == 2) {
+      tc::ld16(tm + lanes + 256 + 96, z);
+      atomicAdd(grad + (row < 64 ? OFF_B2 + row : OFF_B1 + row - 64), z[0]);
     }
   }
   tc::teardown(t, phase, failed, GRAD_TCOLS);
 }
 
 // Adam on the fp32 master parameters; the updated parameter also goes into
-// the training image
-__global__ void k_adam(float *theta, float *m, float *v, const float *grad, int step, float lr, TrainImage *img) {
+// the training image, and the gradient is cleared for the next batch (a
+// clearing of its own was a third launch per batch)
+__global__ void k_adam(float *theta, float *m, float *v, float *grad, int step, float lr, TrainImage *img) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= NP) return;
   const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
   const float gi = grad[i];
+  grad[i] = 0.f;
   const float mi = b1 * m[i] + (1.f - b1) * gi;
   const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
   m[i] = mi;
@@ -583,7 +610,7 @@ int grad_launch(const TrainImage *img, const float *x, const float *t, int n, co
   CKM(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   const int tiles = (n + tc::ROWS - 1) / tc::ROWS;
   const int blocks = tiles < sms ? tiles : sms;
-  k_grad_tc<<<blocks, 128, sizeof(GradSmem), st>>>(img, x, t, n, bt, grad, loss);
+  k_grad_tc<<<blocks, GRAD_THREADS, sizeof(GradSmem), st>>>(img, x, t, n, bt, grad, loss);
   CKM(cudaGetLastError());
   return 0;
 }
@@ -606,9 +633,9 @@ void forward_launch(const float *theta, const float *x, int n, float *y, cudaStr
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  int blocks = tiles < sms ? tiles : sms;
+  int blocks = tiles < FWD_CTAS * sms ? tiles : FWD_CTAS * sms;
   if (blocks < 1) blocks = 1;
-  k_forward_tc<<<blocks, 128, sizeof(tc::Tile), st>>>(theta, x, n, y);
+  k_forward_tc<<<blocks, FWD_THREADS, sizeof(tc::Tile), st>>>(theta, x, n, y);
 }
 }  // namespace mlp
 }  // namespace lbf
@@ -696,6 +723,7 @@ int lbf_mlp_train(const lbf_mlp_train_cfg *cfg, float *theta_io, float *loss_cur
   CKM(cudaMemcpyAsync(theta, theta_io, sizeof(float) * NP, cudaMemcpyHostToDevice, st));
   CKM(cudaMemsetAsync(m, 0, sizeof(float) * NP, st));
   CKM(cudaMemsetAsync(v, 0, sizeof(float) * NP, st));
+  CKM(cudaMemsetAsync(grad, 0, sizeof(float) * NP, st));
   CKM(cudaMemsetAsync(loss, 0, sizeof(double) * (size_t)cfg->epochs, st));
   {
     int rc = image_init(theta, img, st);
@@ -711,7 +739,6 @@ int lbf_mlp_train(const lbf_mlp_train_cfg *cfg, float *theta_io, float *loss_cur
     while (host_gcd(a, (unsigned long long)n) != 1ull) a += 2;
     const unsigned long long b = host_splitmix(h) % (unsigned long long)n;
     for (long long k = 0; k < per_epoch; ++k) {
-      CKM(cudaMemsetAsync(grad, 0, sizeof(float) * NP, st));
       Batch bt{k * B, n, a % (unsigned long long)n, b, host_splitmix(h + (unsigned long long)k),
                (float)cfg->noise};
       int rc = grad_launch(img, x, y, B, bt, grad, loss + ep, st);
