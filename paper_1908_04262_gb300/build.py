@@ -1,8 +1,6 @@
 """Build the CUDA library ``_build/liblbf.so`` for sm_103a with nvcc.
 
-Each translation unit compiles in parallel; the FP64 kernels compile without
-fused multiply-add contraction so that they round like the plain CPU
-reference arithmetic they are compared with.
+Each translation unit compiles in parallel.
 """
 from __future__ import annotations
 
@@ -20,7 +18,7 @@ ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 COMMON = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr",
           "-I", os.path.join(ROOT, "include")]
 UNITS = {
-    "k_f64.cu": ["--fmad=false"],
+    "k_f64.cu": [],
     "k_f32.cu": [],
     "k_f16.cu": [],
     "k_bf16.cu": [],

@@ -34,9 +34,7 @@ __device__ __forceinline__ typename ST<S>::R sum_out_f(const Params &p, const Ce
   for (int i = 0; i < Lat<D>::Q; ++i) {
     const R v = ld(f, slot_out<D>(p, c, n, i, par), fshift<S, D>(p, i));
     rho += v;
-    jx += v * (R)Lat<D>::cx(i);
-    jy += v * (R)Lat<D>::cy(i);
-    jz += v * (R)Lat<D>::cz(i);
+    add_flux<D, R>(i, v, jx, jy, jz);
   }
   if (u) {
     u[0] = (jx - (R)0.5 * rho * PV(R, ax)) / rho;

@@ -90,6 +90,39 @@ __device__ __forceinline__ R cubic_root_in(R b, R c, R d, R lo, R hi) {
   return a;
 }
 
+// The root in [lo, hi] of the decreasing cubic ((a + b) a + c) a + d, in
+// double: the value in double, the slope and the quotient of each step in
+// single precision (a relative 1e-7 of a step that shrinks by as much every
+// time), kept inside the bracket: three or four rounds.  The closed form's
+// FP64 divisions, square root, acos and three cosines, once per branch of
+// the cut, were most of the FP64 geometry (40^3, 2,338 interface cells: 215
+// us a launch; 65 now with the dealt cuts, k_geometry).
+__device__ __forceinline__ double cubic_root_bracketed(double b, double c, double d, double lo, double hi) {
+  const float bf = (float)b, cf = (float)c, df = (float)d;
+  const float lf = (float)lo, hf = (float)hi;
+  float s = 0.5f * (lf + hf);
+#pragma unroll
+  for (int it = 0; it < 4; ++it) {
+    const float v = ((s + bf) * s + cf) * s + df, g = (3.f * s + 2.f * bf) * s + cf;
+    s = fminf(fmaxf(s - v / g, lf), hf);
+  }
+  double a = s >= lf && s <= hf ? (double)s : 0.5 * (lo + hi);
+  a = a < lo ? lo : (a > hi ? hi : a);
+  for (int it = 0; it < 100; ++it) {
+    const double v = ((a + b) * a + c) * a + d;
+    if (v > 0.0) lo = a; else hi = a;
+    const float af = (float)a;
+    double an = a - (double)((float)v / ((3.f * af + 2.f * bf) * af + cf));
+    if (!(an >= lo && an <= hi)) an = 0.5 * (lo + hi);
+    const double step = fabs(an - a);
+    a = an;
+    // what is left is 1e-7 of the step and its square: below the roundoff
+    // of the value (which a bound near it would chase)
+    if (step <= 1e-9) break;
+  }
+  return a;
+}
+
 // plane constant a in [0, 1/2] of the normalised problem: gas fraction V
 // (<= 1/2) of the unit cube below m1 x + m2 y + m3 z = a, m sorted ascending,
 // m1 + m2 + m3 = 1
@@ -108,6 +141,18 @@ __device__ __forceinline__ R plic_a3(R m1, R m2, R m3, R V) {
   if (V < V1) return cbrt((R)6 * m1 * m2 * m3 * V);
   if (V < V2) return (R)0.5 * m1 + sqrt((R)72 * m2 * m3 * V - (R)3 * m1 * m1) / (R)6;
   const R six = (R)6 * m1 * m2 * m3;
+  if constexpr (sizeof(R) == 8) {
+    // one solve for the cubic branches of all lanes
+    const bool over = !(m3 < m12);  // the cut reaches the far corner's planes before m3
+    const R s2 = m1 * m1 + m2 * m2, s3 = m1 * m1 * m1 + m2 * m2 * m2;
+    const R V3 = over ? m12 / ((R)2 * m3) : (m3 * m3 * ((R)3 * m12 - m3) + m1 * m1 * (m1 - (R)3 * m3) + m2 * m2 * (m2 - (R)3 * m3)) / six;
+    const bool low = V < V3;
+    if (over && !low) return m3 * V + (R)0.5 * m12;
+    const R b = low ? (R)-3 * m12 : (R)-1.5;
+    const R c = low ? (R)3 * s2 : (R)1.5 * (s2 + m3 * m3);
+    const R d = low ? -(s3 - six * V) : (R)-0.5 * (s3 + m3 * m3 * m3 - six * V);
+    return cubic_root_bracketed(b, c, d, low ? m2 : m3, low ? (over ? m12 : m3) : (R)0.5);
+  }
   if (m3 < m12) {
     const R V3 = (m3 * m3 * ((R)3 * m12 - m3) + m1 * m1 * (m1 - (R)3 * m3) + m2 * m2 * (m2 - (R)3 * m3)) / six;
     if (V < V3)
@@ -222,14 +267,17 @@ template <int G, class R> __device__ __forceinline__ R group_sum(R v) {
 // lane of each group solves the normal equations and stores the results.
 // Eight blocks of 128 threads per SM (64 registers, no spills) were measured
 // faster than the six that 80 registers allow.
+// FP64 takes 128 registers (four blocks): its pipe is the bound, not the
+// warps in flight, and at 64 the doubles spill.
 constexpr int GEO_LANES = 8;
 
 template <int D, class R>
-__global__ void __launch_bounds__(128, 8) k_geometry(Params p) {
+__global__ void __launch_bounds__(128, sizeof(R) == 4 ? 8 : 4) k_geometry(Params p) {
   constexpr int K = D == 3 ? 5 : 2;
   constexpr int NS = D == 3 ? 27 : 9;
   constexpr int CTR = D == 3 ? 13 : 4;
   constexpr int G = GEO_LANES, CPW = 32 / G, PER = (NS + G - 1) / G;
+  __shared__ R s_cut[4][sizeof(R) == 8 ? CPW : 1][NS];  // fill levels, then offsets, of each group's stencil
   const int lane = threadIdx.x & 31, sub = lane / G, t = lane % G;
   const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int nwarps = (gridDim.x * blockDim.x) >> 5;
@@ -287,12 +335,53 @@ __global__ void __launch_bounds__(128, 8) k_geometry(Params p) {
     const R ign = flat ? (R)0 : (R)1 / gn;
     const R mx = gx * ign, my = gy * ign, mz = gz * ign;
     const Plic<D, R> plic(mx, my, mz);
-    // every thread cuts its own stencil cells (and the centre's holder the centre)
     R sj[PER];
+    if constexpr (sizeof(R) == 4) {
+      // every thread cuts its own stencil cells (and the centre's holder the centre)
 #pragma unroll
-    for (int j = 0; j < PER; ++j) {
-      const int q = t + G * j;
-      sj[j] = (!flat && (act[j] || q == CTR)) ? plic.offset(q == CTR ? ac : a[j]) : (R)0;
+      for (int j = 0; j < PER; ++j) {
+        const int q = t + G * j;
+        sj[j] = (!flat && (act[j] || q == CTR)) ? plic.offset(q == CTR ? ac : a[j]) : (R)0;
+      }
+    } else {
+      // In FP64 the cuts of the group's interface cells (and of the centre) are
+      // dealt to its lanes in turn: about 10 of the 27 stencil cells have one,
+      // so that two rounds of cuts take the place of the four in which every
+      // lane goes through its own cells.  (In single precision that gains 2 of
+      // 24 us in the 128^3 foam but regroups multiply-adds.)
+      unsigned cuts = 0;
+#pragma unroll
+      for (int j = 0; j < PER; ++j) {
+        const int q = t + G * j;
+        const unsigned m = __ballot_sync(0xffffffffu, !flat && (act[j] || q == CTR));
+        cuts |= ((m >> (sub * G)) & ((1u << G) - 1u)) << (G * j);
+        if (q < NS) s_cut[threadIdx.x >> 5][sub][q] = q == CTR ? ac : a[j];
+      }
+      __syncwarp();
+      R *sc = s_cut[threadIdx.x >> 5][sub];
+      const int ncut = __popc(cuts);
+      for (int k = t; __any_sync(0xffffffffu, k < ncut); k += G) {
+        // the k-th set bit
+        unsigned m = cuts;
+        int j = k, q = 0;
+#pragma unroll
+        for (int h = 16; h > 0; h >>= 1) {
+          const int lo = __popc(m & ((1u << h) - 1u));
+          if (j >= lo) {
+            j -= lo;
+            q += h;
+            m >>= h;
+          }
+        }
+        if (k < ncut) sc[q] = plic.offset(sc[q]);
+      }
+      __syncwarp();
+#pragma unroll
+      for (int j = 0; j < PER; ++j) {
+        const int q = t + G * j;
+        sj[j] = (cuts >> q & 1u) ? sc[q < NS ? q : 0] : (R)0;
+      }
+      __syncwarp();
     }
     const R s0 = __shfl_sync(0xffffffffu, sj[CJ], sub * G + CT);
     // local frame (t1, t2, m)

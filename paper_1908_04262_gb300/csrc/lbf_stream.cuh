@@ -152,9 +152,7 @@ __global__ void __launch_bounds__(128) k_exchange(Params p) {
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
       rho += fo[i];
-      jx += fo[i] * (R)Lat<D>::cx(i);
-      jy += fo[i] * (R)Lat<D>::cy(i);
-      jz += fo[i] * (R)Lat<D>::cz(i);
+      add_flux<D, R>(i, fo[i], jx, jy, jz);
       if (i > 0) {
         const int tn = post_type(fn[i]);
         if (tn == T_LIQ || tn == T_IFC)
@@ -286,8 +284,8 @@ __device__ __forceinline__ void relax_store(const Params &p, const Cell &c, long
     for (int j = 0; j < NP; ++j) {
       const int i = 2 * j + 1, k = i + 1;
       const R w = (R)Lat<D>::w(i);
-      const R eu = (R)Lat<D>::cx(i) * ux + (R)Lat<D>::cy(i) * uy + (R)Lat<D>::cz(i) * uz;
-      const R ea = (R)Lat<D>::cx(i) * ax + (R)Lat<D>::cy(i) * ay + (R)Lat<D>::cz(i) * az;
+      const R eu = edot<D, R>(i, ux, uy, uz);
+      const R ea = edot<D, R>(i, ax, ay, az);
       const R fe_even = w * rho * (base + (R)4.5 * eu * eu), fe_odd = w * rho * (R)3 * eu;
       const R f_even = (R)0.5 * (fi[i] + fi[k]), f_odd = (R)0.5 * (fi[i] - fi[k]);
       const R Fe = w * ((R)9 * eu * ea - (R)3 * ua), Fo = w * (R)3 * ea;  // per unit rho
@@ -360,8 +358,8 @@ __device__ __forceinline__ void relax_store(const Params &p, const Cell &c, long
     for (int i = 1; i < Q; i += 2) {
       const int k = i + 1;
       const R w = (R)Lat<D>::w(i);
-      const R eu = (R)Lat<D>::cx(i) * ux + (R)Lat<D>::cy(i) * uy + (R)Lat<D>::cz(i) * uz;
-      const R ea = (R)Lat<D>::cx(i) * ax + (R)Lat<D>::cy(i) * ay + (R)Lat<D>::cz(i) * az;
+      const R eu = edot<D, R>(i, ux, uy, uz);
+      const R ea = edot<D, R>(i, ax, ay, az);
       const R fe_even = w * rho * (base + (R)4.5 * eu * eu), fe_odd = w * rho * (R)3 * eu;
       const R f_even = (R)0.5 * (fi[i] + fi[k]), f_odd = (R)0.5 * (fi[i] - fi[k]);
       const R even = f_even - (f_even - fe_even) * om + w * ge * ((R)9 * eu * ea - (R)3 * ua);
@@ -378,9 +376,8 @@ __device__ __forceinline__ void relax_store(const Params &p, const Cell &c, long
     const R fr = ((R)1 - (R)0.5 * om) * rho;
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
-      const R ex = (R)Lat<D>::cx(i), ey = (R)Lat<D>::cy(i), ez = (R)Lat<D>::cz(i);
-      const R eu = ex * ux + ey * uy + ez * uz;
-      const R ea = ex * ax + ey * ay + ez * az;
+      const R eu = edot<D, R>(i, ux, uy, uz);
+      const R ea = edot<D, R>(i, ax, ay, az);
       const R fe = (R)Lat<D>::w(i) * rho * (base + eu * ((R)3 + eu * (R)4.5));
       const R F = (R)3 * (ea - ua) + (R)9 * eu * ea;
       st(plane(f, p, dir_out<D>(i, 1 - PAR)), cell_out<D>(p, c, i, 1 - PAR),
@@ -397,7 +394,7 @@ __device__ __forceinline__ void relax_store(const Params &p, const Cell &c, long
 #pragma unroll
     for (int i = 1; i < Q; i += 2) {
       const int k = i + 1;
-      const R eu = (R)Lat<D>::cx(i) * ux + (R)Lat<D>::cy(i) * uy + (R)Lat<D>::cz(i) * uz;
+      const R eu = edot<D, R>(i, ux, uy, uz);
       const R wr = (R)Lat<D>::w(i) * rho;
       const R even = wr * (base + (R)4.5 * eu * eu), odd = (R)3 * wr * eu;
       st(plane(f, p, dir_out<D>(i, 1 - PAR)), cell_out<D>(p, c, i, 1 - PAR), fi[i] - (fi[i] - (even + odd)) * om, fshift<S, D>(p, i));
@@ -597,9 +594,7 @@ __device__ __forceinline__ int interface_cell(const Params &p, const Cell &c, lo
 #pragma unroll
   for (int i = 0; i < Q; ++i) {
     rho += fi[i];
-    jx += fi[i] * (R)Lat<D>::cx(i);
-    jy += fi[i] * (R)Lat<D>::cy(i);
-    jz += fi[i] * (R)Lat<D>::cz(i);
+    add_flux<D, R>(i, fi[i], jx, jy, jz);
   }
   const R irho = (R)1 / rho;
   const R ux = (jx + (R)0.5 * rho * PV(R, ax)) * irho;
