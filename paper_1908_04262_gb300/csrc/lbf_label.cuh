@@ -92,7 +92,13 @@ static __global__ void k_label_prep(Params p) {
 
 // union-find tiles: the local pass joins gas cells of one tile in shared
 // memory, the merge pass joins tiles across their faces in global memory
-constexpr int TILE_THREADS = 1024;  // one thread per cell of a tile, one x-row per warp
+// blocks of the tile loops: half a tile each for the local and compress
+// passes (two rows per warp; four blocks per SM cover more of their
+// latencies), a thread per cell for the merge pass (101 x 96 x 99, 60
+// bubbles: local 24.8 us with 1024 threads, 20.5 with 512; compress 9.8 and
+// 8.1; merge 24.7 and 28.7.  Loading all of a cell's far flags before the
+// first test made the merge 32: most links end at the claimed check.)
+constexpr int TILE_THREADS = 512, MERGE_THREADS = 1024;
 
 // parents only ever point to smaller indices, so a chain has at most TN
 // links; the caps below are never reached by a consistent forest
@@ -190,11 +196,21 @@ __global__ void __launch_bounds__(TILE_THREADS) k_uf_local(Params p) {
       rfirst = TN;
     }
     __syncthreads();
-    // row masks, runs
-    for (int r = warp; r < NR; r += TILE_THREADS / 32) {
+    // row masks, runs (every row's flags loaded before any is used)
+    constexpr int RPW = NR / (TILE_THREADS / 32);  // rows per warp
+    uint8_t fl[RPW];
+#pragma unroll
+    for (int k = 0; k < RPW; ++k) {
+      const int r = warp + k * (TILE_THREADS / 32);
+      const int x = x0 + lane, y = y0 + r % TY, z = z0 + r / TY;
+      fl[k] = x < p.nx && y < p.ny && z < p.nz ? p.flags[x + nx * y + nxy * z] : (uint8_t)T_WALL;
+    }
+#pragma unroll
+    for (int k = 0; k < RPW; ++k) {
+      const int r = warp + k * (TILE_THREADS / 32);
       const int x = x0 + lane, y = y0 + r % TY, z = z0 + r / TY;
       const bool inside = x < p.nx && y < p.ny && z < p.nz;
-      const bool gas = inside && post_type(p.flags[x + nx * y + nxy * z]) == T_GAS;
+      const bool gas = inside && post_type(fl[k]) == T_GAS;
       const unsigned m = __ballot_sync(0xffffffffu, gas), in = __ballot_sync(0xffffffffu, inside);
       if (lane == 0) {
         rowm[r] = m;
@@ -282,11 +298,15 @@ __global__ void __launch_bounds__(TILE_THREADS) k_uf_local(Params p) {
   }
 }
 
+// a coordinate one cell outside the lattice at most, wrapped (three runtime
+// remainders per crossing link were a good part of the merge pass)
+__device__ __forceinline__ int wrap1(int x, int n) { return x < 0 ? x + n : (x >= n ? x - n : x); }
+
 // one block per tile: join gas components across tile faces (and the
 // periodic boundary).  Two all-gas tiles are joined by one union of their
 // roots; otherwise every crossing link of a gas cell is joined.
 template <int D>
-__global__ void __launch_bounds__(TILE_THREADS) k_uf_merge(Params p) {
+__global__ void __launch_bounds__(MERGE_THREADS) k_uf_merge(Params p) {
   constexpr int TX = Tile<D>::TX, TY = Tile<D>::TY, TZ = Tile<D>::TZ, TN = TX * TY * TZ;
   if (label_fast(p)) return;
   const int mode = label_mode(p);
@@ -324,7 +344,7 @@ __global__ void __launch_bounds__(TILE_THREADS) k_uf_merge(Params p) {
     __syncthreads();
     if (mode == LABEL_ADDED && !near_dirty) continue;
     bool ok = true;
-    for (int t = threadIdx.x; t < TN; t += TILE_THREADS) {
+    for (int t = threadIdx.x; t < TN; t += MERGE_THREADS) {
       const int lx = t % TX, ly = (t / TX) % TY, lz = t / (TX * TY);
       const int x = x0 + lx, y = y0 + ly, z = z0 + lz;
       if (x >= p.nx || y >= p.ny || z >= p.nz) continue;
@@ -347,7 +367,7 @@ __global__ void __launch_bounds__(TILE_THREADS) k_uf_merge(Params p) {
         const int ns = nst[oi];
         if (ns == 0) continue;
         if (own == 1 && ns == 1 && claimed[oi]) continue;
-        const long long m = at_far(p, ax, ay, az);
+        const long long m = wrap1(ax, p.nx) + nx * wrap1(ay, p.ny) + nxy * wrap1(az, p.nz);
         if (post_type(p.flags[m]) != T_GAS) continue;
         if (own == 1 && ns == 1 && atomicExch(&claimed[oi], 1)) continue;
         // representatives: the parents the local pass left (any ancestor
@@ -465,18 +485,6 @@ static __global__ void k_sort_roots(Params p) {
     // forest is current again
     if (p.forest_stale) *p.forest_stale = 0;
   }
-}
-
-__device__ __forceinline__ int root_index(const int *roots, int cnt, int r) {
-  int lo = 0, hi = cnt;
-  while (lo < hi) {
-    const int mid = (lo + hi) >> 1;
-    if (roots[mid] < r)
-      lo = mid + 1;
-    else
-      hi = mid;
-  }
-  return (lo < cnt && roots[lo] == r) ? lo : -1;
 }
 
 __device__ __forceinline__ void hash_insert(const Params &p, unsigned long long key) {

@@ -45,32 +45,41 @@ int fail(int code, const char *msg) {
   return code;
 }
 
-// final labels: gas cells get the rank of their root among the sorted roots,
-// interface cells the smallest label of their gas neighbours, others -1
+// final labels: gas cells get the rank of their root among the sorted roots
+// (k_sort_roots left it at the root, in rlabel), interface cells the
+// smallest label of their gas neighbours, others -1.  The neighbours' flags
+// are loaded together, then the parents, then the ranks: three latencies in
+// turn, where a branch and a binary search per neighbour followed one
+// another (101 x 96 x 99, 60 bubbles: 22.4 -> 10.3 us)
 template <int D>
-__global__ void k_cc_label(Params p, int32_t *label, int32_t *count) {
+__global__ void __launch_bounds__(128) k_cc_label(Params p, int32_t *label, int32_t *count) {
   Cell c;
   const bool inr = grid_cell(p, c);
-  const int cnt = *p.tnew.count;
   if (inr) {
-    const long long n = c.n;
+    const int n = c.n;
     const int t = ftype(p.flags[n]);
     int k = -1;
     if (t == T_GAS) {
-      k = root_index(p.roots, cnt, p.parent[n]);
+      k = p.rlabel[p.parent[n]];
     } else if (t == T_IFC) {
+      int m[Lat<D>::Q];
+      uint8_t fn[Lat<D>::Q];
 #pragma unroll
       for (int i = 1; i < Lat<D>::Q; ++i) {
-        const long long m = nb<D>(p, c, i);
-        if (ftype(p.flags[m]) == T_GAS) {
-          const int r = root_index(p.roots, cnt, p.parent[m]);
-          if (r >= 0 && (k < 0 || r < k)) k = r;
-        }
+        m[i] = nb<D>(p, c, i);
+        fn[i] = p.flags[m[i]];
       }
+#pragma unroll
+      for (int i = 1; i < Lat<D>::Q; ++i) m[i] = ftype(fn[i]) == T_GAS ? p.parent[m[i]] : -1;
+#pragma unroll
+      for (int i = 1; i < Lat<D>::Q; ++i) m[i] = m[i] >= 0 ? p.rlabel[m[i]] : -1;
+#pragma unroll
+      for (int i = 1; i < Lat<D>::Q; ++i)
+        if (m[i] >= 0 && (k < 0 || m[i] < k)) k = m[i];
     }
     label[n] = k;
   }
-  if (blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.x == 0) *count = *p.err ? -1 : cnt;
+  if (blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.x == 0) *count = *p.err ? -1 : *p.tnew.count;
 }
 
 __global__ void k_cc_reset(Scratch *s) {
@@ -91,6 +100,9 @@ int run(Scratch *s, const uint8_t *type, int nx, int ny, int nz, int32_t *label,
   p.flags = const_cast<uint8_t *>(type);
   p.parent = s->parent;
   p.lsize = s->lsize;
+  // the component sizes of the tile-local pass are not needed here: the
+  // ranks of the roots take their place once the forest is built
+  p.rlabel = s->lsize;
   p.tstat = s->tstat;
   p.troot = s->troot;
   p.roots = s->roots;
@@ -104,7 +116,7 @@ int run(Scratch *s, const uint8_t *type, int nx, int ny, int nz, int32_t *label,
   const dim3 rg((unsigned)((nx + b - 1) / b), (unsigned)ny, (unsigned)nz);
   k_cc_reset<<<1, 1, 0, st>>>(s);
   k_uf_local<D><<<tg, TILE_THREADS, 0, st>>>(p);
-  k_uf_merge<D><<<tg, TILE_THREADS, 0, st>>>(p);
+  k_uf_merge<D><<<tg, MERGE_THREADS, 0, st>>>(p);
   k_uf_compress<D><<<tg, TILE_THREADS, 0, st>>>(p);
   k_sort_roots<<<1, 1024, kMaxBubbles * sizeof(int), st>>>(p);
   k_cc_label<D><<<rg, b, 0, st>>>(p, label, count);

@@ -119,12 +119,13 @@ struct OpsImpl final : Ops {
   void label_forest(const Params &p, cudaStream_t s) override {
     const dim3 tg((unsigned)((p.nx + Tile<D>::TX - 1) / Tile<D>::TX), (unsigned)((p.ny + Tile<D>::TY - 1) / Tile<D>::TY),
                   (unsigned)((p.nz + Tile<D>::TZ - 1) / Tile<D>::TZ));
-    // tile loops on a grid of two blocks per SM (a block of the
+    // tile loops on a grid of two or four blocks per SM (a block of the
     // graph's patch steps then costs one short wave)
     const unsigned ntiles = tg.x * tg.y * tg.z;
-    const unsigned g = p.tile_blocks > 0 && (unsigned)p.tile_blocks < ntiles ? (unsigned)p.tile_blocks : ntiles;
+    const unsigned two = p.tile_blocks > 0 ? (unsigned)p.tile_blocks : ntiles;
+    const unsigned gm = two < ntiles ? two : ntiles, g = 2 * two < ntiles ? 2 * two : ntiles;
     k_uf_local<D><<<g, TILE_THREADS, 0, s>>>(p);
-    k_uf_merge<D><<<g, TILE_THREADS, 0, s>>>(p);
+    k_uf_merge<D><<<gm, MERGE_THREADS, 0, s>>>(p);
     k_uf_compress<D><<<g, TILE_THREADS, 0, s>>>(p);
     int P = 1;
     while (P < p.cap) P <<= 1;
