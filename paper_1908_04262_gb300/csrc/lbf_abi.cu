@@ -97,9 +97,9 @@ struct lbf_sim {
   size_t ntiles_alloc = 0;
   unsigned *wmask = nullptr;
   int *rlabel = nullptr;
-  unsigned char *bub_dev = nullptr;   // packed bubble rows: count (16 bytes), then lbf_bubble records
-  unsigned char *bub_host = nullptr;  // pinned staging copy
-  int *err_host = nullptr;            // pinned copy of the sticky error bits
+  unsigned char *bub_host = nullptr;  // page-locked bubble rows: count (16 bytes), then lbf_bubble records
+  int *err_host = nullptr;            // page-locked copy of the sticky error bits: [0] copied by
+                                      // check_device_error, [1] set by the steps
   void *pin[2] = {nullptr, nullptr};  // pinned chunks for host copies of fields
   cudaEvent_t pin_ev[2] = {nullptr, nullptr};
   double *acc = nullptr;
@@ -195,6 +195,7 @@ Params make_params(lbf_sim *s, long long step) {
   p.rmv = s->rmv;
   p.rmlist = s->rmlist;
   p.rank = s->rank;
+  p.err_host = s->err_host + 1;
   p.scan_done = s->scan_done;
   p.clist = s->clist;
   p.ccount = s->ccount;
@@ -641,11 +642,12 @@ int copy_to_host(lbf_sim *s, void *dst, const void *src, size_t bytes) {
   return 0;
 }
 
-int check_device_error(lbf_sim *s) {
-  if (!s->err_host) CK(cudaMallocHost((void **)&s->err_host, sizeof(int)));
-  CK(cudaMemcpyAsync(s->err_host, s->err, sizeof(int), cudaMemcpyDeviceToHost, s->st));
+// stepped: steps ran, and each set its bits in err_host[1] too
+// (k_bubble_update), so that no copy follows the graph
+int check_device_error(lbf_sim *s, bool stepped = false) {
+  if (!stepped) CK(cudaMemcpyAsync(s->err_host, s->err, sizeof(int), cudaMemcpyDeviceToHost, s->st));
   CK(cudaStreamSynchronize(s->st));
-  const int e = *s->err_host;
+  const int e = s->err_host[stepped ? 1 : 0];
   if (e & ERR_CAPACITY) return fail(LBF_ECAPACITY, "more bubbles than bubble_capacity");
   if (e & ERR_NOTCONV) return fail(LBF_ENOTCONV, "union-find iteration cap reached");
   if (e & ERR_HASH) return fail(LBF_ECAPACITY, "bubble overlap table full");
@@ -1062,6 +1064,11 @@ int lbf_create(const lbf_config *cfg, lbf_sim **out) {
     return fail(rc, msg);
   }
   s->n_state_allocs = s->allocs.size();
+  if (cudaMallocHost((void **)&s->err_host, 2 * sizeof(int)) != cudaSuccess) {
+    lbf_destroy(s);
+    return fail(LBF_ENOMEM, "cudaMallocHost");
+  }
+  s->err_host[0] = s->err_host[1] = 0;
   // scratch, not part of a checkpoint
   rc = dalloc(s, &s->rank, s->cap);
   if (!rc) rc = dalloc(s, &s->rmlist, s->cap);
@@ -1189,7 +1196,7 @@ int lbf_step(lbf_sim *s, int nsteps) {
       ++k;
     }
   }
-  return check_device_error(s);
+  return check_device_error(s, nsteps > 0);
 }
 
 long long lbf_step_count(const lbf_sim *s) { return s ? s->step : -1; }
@@ -1384,6 +1391,7 @@ int lbf_checkpoint_load(lbf_sim *s, const void *src, size_t bytes) {
   }
   CK(cudaMemsetAsync(s->ccount, 0x7f, sizeof(int), s->st));  // contacts unknown
   CK(cudaStreamSynchronize(s->st));
+  s->err_host[1] = 0;
   s->step = h.step;
   s->walled = h.walled != 0 && all_faces_walled(s);
   s->queue.swap(q);
@@ -1393,31 +1401,18 @@ int lbf_checkpoint_load(lbf_sim *s, const void *src, size_t bytes) {
 
 int lbf_bubbles(lbf_sim *s, lbf_bubble *out, int capacity, int *count) {
   if (!s || !count || capacity < 0 || (capacity > 0 && !out)) return fail(LBF_EINVAL, "bad arguments");
-  // rows packed on the device, then one copy into pinned staging memory
+  // rows packed by a kernel straight into page-locked host memory: one
+  // launch and one wait (a copy of the first rows, and a second one past 64,
+  // had followed the kernel)
   const int rows = std::min(capacity, s->cap);
-  const size_t bytes = 16 + sizeof(lbf_bubble) * (size_t)rows;
-  if (!s->bub_dev) {
-    int rc = dev_alloc(s, (void **)&s->bub_dev, 16 + sizeof(lbf_bubble) * (size_t)s->cap);
-    if (rc) return rc;
-    CK(cudaMallocHost((void **)&s->bub_host, 16 + sizeof(lbf_bubble) * (size_t)s->cap));
-  }
-  lbf::pack_bubbles_launch(s->tab[s->step & 1], s->bub_dev, rows, s->cap, s->st);
+  if (!s->bub_host) CK(cudaMallocHost((void **)&s->bub_host, 16 + sizeof(lbf_bubble) * (size_t)s->cap));
+  lbf::pack_bubbles_launch(s->tab[s->step & 1], s->bub_host, rows, s->cap, s->st);
   CK(cudaGetLastError());
-  // the header and the first rows in one copy; the rest only when present
-  constexpr int kFirst = 64;
-  const size_t first = std::min(bytes, 16 + sizeof(lbf_bubble) * (size_t)kFirst);
-  CK(cudaMemcpyAsync(s->bub_host, s->bub_dev, first, cudaMemcpyDeviceToHost, s->st));
   CK(cudaStreamSynchronize(s->st));
   int nb = 0;
   std::memcpy(&nb, s->bub_host, sizeof(int));
   *count = nb;
   const int k = std::min(nb, rows);
-  if (k > kFirst) {
-    const size_t off = 16 + sizeof(lbf_bubble) * (size_t)kFirst;
-    CK(cudaMemcpyAsync(s->bub_host + off, s->bub_dev + off, sizeof(lbf_bubble) * (size_t)(k - kFirst),
-                       cudaMemcpyDeviceToHost, s->st));
-    CK(cudaStreamSynchronize(s->st));
-  }
   if (k > 0) std::memcpy(out, s->bub_host + 16, sizeof(lbf_bubble) * (size_t)k);
   return 0;
 }

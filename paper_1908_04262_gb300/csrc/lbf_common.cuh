@@ -154,6 +154,7 @@ struct Params {
   double *led;                   // 8 ledger accumulators
   unsigned long long *fluid_updates;
   int *err;
+  int *err_host;  // page-locked host copy (bits set by the step)
   // what the conversion of this step did to the gas cells: 0 nothing (the
   // forest of the last labelling is still exact), 1 added some only (the
   // components can only grow or merge: the touched tiles, marked in

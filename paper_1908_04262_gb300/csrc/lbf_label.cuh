@@ -563,10 +563,17 @@ __device__ __forceinline__ void relabel_all(const Params &p, double *wbuf) {
 // Group bookkeeping lives in shared memory when there are at most
 // K10_SMEM old + new bubbles, in the global scratch arrays otherwise.
 constexpr int K10_SMEM = 512;
+// the step's sticky error bits, if any, to the host's copy
+__device__ __forceinline__ void tell_host(const Params &p) {
+  if (threadIdx.x != 0) return;
+  const int e = *(volatile int *)p.err;
+  if (e) atomicOr_system(p.err_host, e);
+}
 static __device__ __forceinline__ void update_kept(const Params &p);
 static __global__ void __launch_bounds__(1024) k_bubble_update(Params p) {
   if (label_fast(p)) {
     update_kept(p);
+    tell_host(p);
     return;
   }
   __shared__ int sfresh[1024];
@@ -702,6 +709,7 @@ static __global__ void __launch_bounds__(1024) k_bubble_update(Params p) {
     *p.hcount = 0;
     *p.nroots = 0;
     if (p.gas_dirty) *p.gas_dirty = 0;
+    tell_host(p);  // (this block's own bits were set barriers ago)
   }
   // the old table is the next step's new table: clear its accumulators
   for (int k = tid; k < p.cap; k += nt) {

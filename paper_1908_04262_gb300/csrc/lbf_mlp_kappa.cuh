@@ -96,7 +96,12 @@ __global__ void __launch_bounds__(MLP_THREADS) k_mlp_kappa(Params p, const tc::I
       }
       __syncthreads();
     }
-    if (failed && tid == 0) atomicOr(p.err, ERR_TC_WAIT);
+    if (failed && tid == 0) {
+      // this runs beside the bubble update, which may already have told the
+      // host the bits of this step
+      atomicOr(p.err, ERR_TC_WAIT);
+      atomicOr_system(p.err_host, ERR_TC_WAIT);
+    }
     tc::teardown(t, phase, failed);
   }
 }
