@@ -469,14 +469,29 @@ __global__ void __launch_bounds__(128) k_gen_quadrics(const double *par, int n, 
   out[i] = q;
 }
 
+// one row of six sub-points in double (out of line: inlined, its FP64 set-up
+// was hoisted into every row and the kernel took 600 us for 98,304 samples)
+__device__ __noinline__ int row_in_double(const double *P, const Quadric &q, int ox, int oy, int oz, int ky, int kz) {
+  int row = 0;
+  const double cx = P[16] + ox - P[0], ddy = P[17] + oy - P[1] + (ky + 0.5) / 6 - 0.5,
+               ddz = P[18] + oz - P[2] + (kz + 0.5) / 6 - 0.5;
+  for (int kx = 0; kx < 6; ++kx) {
+    const double dx = cx + (kx + 0.5) / 6 - 0.5;
+    const double f = q.A64[0] * dx * dx + q.A64[1] * ddy * ddy + q.A64[2] * ddz * ddz +
+                     2 * (q.A64[3] * dx * ddy + q.A64[4] * dx * ddz + q.A64[5] * ddy * ddz);
+    row += f < 1.0;
+  }
+  return row;
+}
+
 // Fill levels (fraction of 6^3 sub-points that are liquid), axes as they
 // are.  One warp per sample, one lane per stencil cell; a sub-point is
 // inside where F < 0.  Single precision decides wherever |F| exceeds its
 // error bound; the few sub-points within it (about one row in 1e4) are
 // evaluated in double like all of them used to be, so the counts are the
 // same.  With 5,832 double evaluations a sample on an FP64 pipe of 1/64 rate
-// a whole generation of 100,000 samples took 12.7 ms; it takes 1.1 ms, 0.6 of
-// them here, every row bit for bit as before.
+// a whole generation of 100,000 samples took 12.7 ms; it takes 0.63 ms, 0.14
+// of them here, every row bit for bit as before.
 __global__ void __launch_bounds__(128) k_gen_fill(const double *par, const Quadric *quad, int n, float *x) {
   const int lane = threadIdx.x & 31;
   const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nwarps = (gridDim.x * blockDim.x) >> 5;
@@ -506,16 +521,7 @@ __global__ void __launch_bounds__(128) k_gen_fill(const double *par, const Quadr
           least = fminf(least, fabsf(F));
         }
         if (!(least > tol)) {  // (a shape that is not finite too)
-          const double *P = par + (size_t)i * 20;
-          row = 0;
-          const double cx = P[16] + ox - P[0], ddy = P[17] + oy - P[1] + (ky + 0.5) / 6 - 0.5,
-                       ddz = P[18] + oz - P[2] + (kz + 0.5) / 6 - 0.5;
-          for (int kx = 0; kx < 6; ++kx) {
-            const double dx = cx + (kx + 0.5) / 6 - 0.5;
-            const double f = q.A64[0] * dx * dx + q.A64[1] * ddy * ddy + q.A64[2] * ddz * ddz +
-                             2 * (q.A64[3] * dx * ddy + q.A64[4] * dx * ddz + q.A64[5] * ddy * ddz);
-            row += f < 1.0;
-          }
+          row = row_in_double(par + (size_t)i * 20, q, ox, oy, oz, ky, kz);
         }
         in += row;
       }
