@@ -37,28 +37,82 @@ int fail(int code, const char *msg) {
 // tensor-memory columns hold at 128 each) of 256 threads (two per row, half
 // the columns each) instead of one of 128.  What then bounds it is the
 // special-function unit, two results for each of the 128 SiLUs of a row
-// (27 us at 503,117 rows).  Measured there: 208 -> 68 us.
+// (27 us at 503,117 rows).  Measured there: 208 -> 68 us, and 50 with the
+// inputs staged as below.
 constexpr int FWD_THREADS = 256, FWD_CTAS = 4;
+//
+// The inputs of a full tile are 13,824 consecutive bytes: one bulk copy
+// brings them into shared memory while the tile before is worked on, and
+// each thread packs half a row from there (27 words apart, no bank
+// conflicts) into two 16-byte pieces of the operand.  The last, partial tile
+// and inputs that do not start on 16 bytes are gathered with plain loads.
+struct __align__(128) FwdSmem {
+  tc::Tile t;
+  float x[tc::ROWS * 27];
+  uint64_t mbar;
+};
 __global__ void __launch_bounds__(FWD_THREADS, FWD_CTAS) k_forward_tc(const float *theta, const float *x, int n, float *y) {
   extern __shared__ __align__(128) unsigned char tsm[];
-  tc::Tile &t = *reinterpret_cast<tc::Tile *>(tsm);
+  FwdSmem &s = *reinterpret_cast<FwdSmem *>(tsm);
+  tc::Tile &t = s.t;
+  constexpr uint32_t XBYTES = tc::ROWS * 27 * 4;
+  const int tiles = (n + tc::ROWS - 1) / tc::ROWS, full = (reinterpret_cast<uintptr_t>(x) & 15) == 0 ? n / tc::ROWS : 0;
+  if (threadIdx.x == 0) {
+    tc::mbar_init(&s.mbar, 1);
+    if ((int)blockIdx.x < full) {
+      tc::expect_bytes(&s.mbar, XBYTES);
+      tc::bulk_copy(s.x, x + (long long)blockIdx.x * (tc::ROWS * 27), XBYTES, &s.mbar);
+    }
+  }
   tc::pack_image(t.net, theta);
   tc::setup(t, tc::TCOLS);
-  uint32_t phase = 0;
-  bool failed = false;
-  const int tiles = (n + tc::ROWS - 1) / tc::ROWS;
+  uint32_t phase = 0, xphase = 0;  // parities of the MMAs' and of the input copies' next phase
+  bool failed = false, flying = (int)blockIdx.x < full;  // flying: an input copy is under way
   for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
     const long long row0 = (long long)tile * tc::ROWS;
     const int rows = (int)min((long long)tc::ROWS, (long long)n - row0);
-    const float *xt = x + row0 * 27;
-    for (int e = threadIdx.x; e < tc::ROWS * 27; e += blockDim.x) {
-      const int r = e / 27, k = e - 27 * r;
-      tc::put_x(t, r, k, r < rows ? xt[e] : 0.f);
-    }
     float yv = __int_as_float(0x7fc00000);
+    if (!failed && tile < full) {
+      const bool ok = tc::mbar_wait(&s.mbar, xphase);
+      failed = __syncthreads_or(!ok) != 0;
+      if (!failed) {
+        xphase ^= 1u;
+        flying = false;
+        // thread: 16 of the 32 inputs (27 and five zeros) of one row
+        const int r = threadIdx.x & (tc::ROWS - 1), k0 = 16 * (threadIdx.x >> 7);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          float v[8];
+#pragma unroll
+          for (int e = 0; e < 8; ++e) {
+            const int k = k0 + 8 * h + e;
+            v[e] = k < 27 ? s.x[27 * r + k] : 0.f;
+          }
+          const uint4 q = make_uint4(pack2(v[0], v[1]), pack2(v[2], v[3]), pack2(v[4], v[5]), pack2(v[6], v[7]));
+          *reinterpret_cast<uint4 *>(reinterpret_cast<unsigned char *>(t.a1) + tc::kofs(r, k0 + 8 * h, 32)) = q;
+        }
+        __syncthreads();  // the staged inputs are read: the next tile's may come
+        const int next = tile + (int)gridDim.x;
+        if (next < full) {
+          flying = true;
+          if (threadIdx.x == 0) {
+            tc::expect_bytes(&s.mbar, XBYTES);
+            tc::bulk_copy(s.x, x + (long long)next * (tc::ROWS * 27), XBYTES, &s.mbar);
+          }
+        }
+      }
+    } else if (!failed) {
+      const float *xt = x + row0 * 27;
+      for (int e = threadIdx.x; e < tc::ROWS * 27; e += blockDim.x) {
+        const int r = e / 27, k = e - 27 * r;
+        tc::put_x(t, r, k, r < rows ? xt[e] : 0.f);
+      }
+    }
     if (!failed) failed = !tc::forward_tile<FWD_THREADS>(t, phase, yv);
     if ((int)threadIdx.x < rows) y[row0 + threadIdx.x] = yv;
   }
+  // a copy still under way (after a wait that gave up) is given one more wait
+  if (flying && threadIdx.x == 0) (void)tc::mbar_wait(&s.mbar, xphase);
   tc::teardown(t, phase, failed);
 }
 
@@ -641,7 +695,12 @@ void forward_launch(const float *theta, const float *x, int n, float *y, cudaStr
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   int blocks = tiles < FWD_CTAS * sms ? tiles : FWD_CTAS * sms;
   if (blocks < 1) blocks = 1;
-  k_forward_tc<<<blocks, FWD_THREADS, sizeof(tc::Tile), st>>>(theta, x, n, y);
+  static int attr_dev = -1;
+  if (attr_dev != dev) {
+    cudaFuncSetAttribute(k_forward_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(FwdSmem));
+    attr_dev = dev;
+  }
+  k_forward_tc<<<blocks, FWD_THREADS, sizeof(FwdSmem), st>>>(theta, x, n, y);
 }
 }  // namespace mlp
 }  // namespace lbf
