@@ -19,6 +19,7 @@ COMMON = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "--expt-relax
           "-I", os.path.join(ROOT, "include")]
 UNITS = {
     "k_f64.cu": [],
+    "k_f64_net.cu": ["--fmad=false"],
     "k_f32.cu": [],
     "k_f16.cu": [],
     "k_bf16.cu": [],

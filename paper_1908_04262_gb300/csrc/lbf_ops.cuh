@@ -150,7 +150,9 @@ struct OpsImpl final : Ops {
     // up to two CTAs of 128 cells per SM (list_blocks holds 4 per SM);
     // each holds 128 of the SM's 512 tensor-memory columns, and no more
     // than four fit on an SM by their shared memory
-    if (D == 3)
+    if constexpr (D == 3 && sizeof(R) == 8)
+      mlp_kappa_f64(p, img, p.list_blocks / 2, s);
+    else if (D == 3)
       k_mlp_kappa<D, R><<<p.list_blocks / 2, MLP_THREADS, sizeof(tc::Tile), s>>>(p, (const tc::Image *)img);
   }
   void mlp_harvest(const Params &p, float *x, float *y, int *cells, int cap, int *count, cudaStream_t s) override {

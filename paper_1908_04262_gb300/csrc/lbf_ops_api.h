@@ -13,6 +13,9 @@ namespace lbf {
 // network's bulk copy) ran past its bound
 constexpr int ERR_TC_WAIT = 8;
 
+// the network kernel of the double-precision form (a unit of its own)
+void mlp_kappa_f64(const Params &p, const void *img, int blocks, cudaStream_t s);
+
 struct Ops {
   virtual ~Ops() {}
   virtual void init_fill(const Params &p, int par, double h, cudaStream_t s) = 0;
