@@ -33,10 +33,9 @@ sys.path.insert(0, ROOT)
 
 METRIC = "MLUPS (D3Q19 FSLBM + D3Q7 ADE) and % HBM roofline; FP16+learned-κ vs FP32 plain"
 WORKLOAD = "3D D3Q19 FSLBM + D3Q7 ADE, 128^3, FP32 storage, 8 bubbles (R 4-6), power-law n=0.6, disjoining on"
-# label sync 1, exchange 1, sweep 2, conversion 4, labelling check, root scan and choice 3, union-find 4,
-# relabel 1, label patch 1, bubble update 2, geometry 1, disjoining 1 (one of the two labelling branches
-# returns at once)
-KERNELS_PER_STEP = 21
+# label sync 1, exchange 1, sweep 2, conversion 4, labelling check and root scan 2, union-find 4 (they
+# return at once in a patched step), patch or relabel 1, bubble update 1, geometry 1, disjoining 1
+KERNELS_PER_STEP = 18
 
 
 def parse():
@@ -124,7 +123,7 @@ def stop_clocks(proc, path):
 # were profiled
 SWEEP_TRAFFIC_BYTES = 264.1e6
 SWEEP_SOURCES = ("paper_1908_04262_gb300/csrc/lbf_stream.cuh", "paper_1908_04262_gb300/csrc/lbf_common.cuh")
-SWEEP_SOURCES_SHA256_16 = "a6b86d84b81863eb"
+SWEEP_SOURCES_SHA256_16 = "a86b0a7a4451b518"
 
 
 def sweep_traffic():
