@@ -5,10 +5,11 @@
 // Normal: gradient of the fill level over the 3^d stencil with face, edge and
 // corner weights 4, 2, 1, normalised; it points into the liquid.
 // PLIC: the plane n.p = s that leaves liquid fraction alpha on its +n side of
-// the unit cell, inverted in closed form after Scardovelli and Zaleski (2000)
-// (volume of a unit cube cut by a plane: piecewise polynomial in the
-// plane constant; its quadratic branches are solved directly, its cubic
-// branches by the trigonometric formula, then one Newton polish).
+// the unit cell, inverted after Scardovelli and Zaleski (2000) (volume of a
+// unit cube cut by a plane: piecewise polynomial in the plane constant; its
+// quadratic branches are solved directly, its cubic branches in single
+// precision by the trigonometric formula and two Newton steps, in double as
+// depressed cubics by a fixed number of Newton steps, cut_cubic).
 // Curvature: least-squares paraboloid through the PLIC points of the
 // interface cells of the stencil (each cut with the centre normal) in a frame
 // whose third axis is the normal (ridge-regularised normal equations);
@@ -42,85 +43,74 @@ __device__ __forceinline__ float acos_as(float x) {
 }
 
 // real root of a^3 + b a^2 + c a + d = 0 closest to [lo, hi], polished
-template <class R>
-__device__ __forceinline__ R cubic_root_in(R b, R c, R d, R lo, R hi) {
-  const R b3 = b / (R)3;
-  const R P = c - b * b3;
-  const R Qc = (R)2 * b3 * b3 * b3 - b3 * c + d;
-  R best = (R)0.5 * (lo + hi), bestd = (R)1e30;
-  auto consider = [&](R a) {
-    const R dd = a < lo ? lo - a : (a > hi ? a - hi : (R)0);
+// (single precision: the double form solves the cuts otherwise, see
+// cut_cubic)
+__device__ __forceinline__ float cubic_root_in(float b, float c, float d, float lo, float hi) {
+  const float b3 = b / 3.f;
+  const float P = c - b * b3;
+  const float Qc = 2.f * b3 * b3 * b3 - b3 * c + d;
+  float best = 0.5f * (lo + hi), bestd = 1e30f;
+  auto consider = [&](float a) {
+    const float dd = a < lo ? lo - a : (a > hi ? a - hi : 0.f);
     if (dd < bestd) {
       bestd = dd;
       best = a;
     }
   };
-  if (P < (R)0) {
-    const R r = (R)2 * sqrt(-P / (R)3);
-    R arg = (R)3 * Qc / (P * r);
-    arg = arg < (R)-1 ? (R)-1 : (arg > (R)1 ? (R)1 : arg);
-    if constexpr (sizeof(R) == 4) {
-      // the three cosines cos(th - 2 pi k / 3) from one sine and cosine
-      const float th = acos_as(arg) * (1.f / 3.f);
-      float sn, cs;
-      __sincosf(th, &sn, &cs);
-      const float h = 0.8660254037844386f * sn;
-      consider(r * cs - b3);
-      consider(r * (-0.5f * cs + h) - b3);
-      consider(r * (-0.5f * cs - h) - b3);
-    } else {
-      const R th = acos(arg) / (R)3;
-      const R twopi3 = (R)2.0943951023931954923;
-      for (int k = 0; k < 3; ++k) consider(r * cos(th - twopi3 * (R)k) - b3);
-    }
+  if (P < 0.f) {
+    const float r = 2.f * sqrt(-P / 3.f);
+    float arg = 3.f * Qc / (P * r);
+    arg = arg < -1.f ? -1.f : (arg > 1.f ? 1.f : arg);
+    // the three cosines cos(th - 2 pi k / 3) from one sine and cosine
+    const float th = acos_as(arg) * (1.f / 3.f);
+    float sn, cs;
+    __sincosf(th, &sn, &cs);
+    const float h = 0.8660254037844386f * sn;
+    consider(r * cs - b3);
+    consider(r * (-0.5f * cs + h) - b3);
+    consider(r * (-0.5f * cs - h) - b3);
   } else {
-    const R disc = Qc * Qc / (R)4 + P * P * P / (R)27;
-    const R sq = sqrt(disc > (R)0 ? disc : (R)0);
-    consider(cbrt(-Qc / (R)2 + sq) + cbrt(-Qc / (R)2 - sq) - b3);
+    const float disc = Qc * Qc / 4.f + P * P * P / 27.f;
+    const float sq = sqrt(disc > 0.f ? disc : 0.f);
+    consider(cbrt(-Qc / 2.f + sq) + cbrt(-Qc / 2.f - sq) - b3);
   }
-  R a = best < lo ? lo : (best > hi ? hi : best);
+  float a = best < lo ? lo : (best > hi ? hi : best);
   for (int it = 0; it < 2; ++it) {
-    const R fa = ((a + b) * a + c) * a + d;
-    const R fp = ((R)3 * a + (R)2 * b) * a + c;
-    if (fp != (R)0) {
-      const R an = a - fa / fp;
+    const float fa = ((a + b) * a + c) * a + d;
+    const float fp = (3.f * a + 2.f * b) * a + c;
+    if (fp != 0.f) {
+      const float an = a - fa / fp;
       a = an < lo ? lo : (an > hi ? hi : an);
     }
   }
   return a;
 }
 
-// The root in [lo, hi] of the decreasing cubic ((a + b) a + c) a + d, in
-// double: the value in double, the slope and the quotient of each step in
-// single precision (a relative 1e-7 of a step that shrinks by as much every
-// time), kept inside the bracket: three or four rounds.  The closed form's
-// FP64 divisions, square root, acos and three cosines, once per branch of
-// the cut, were most of the FP64 geometry (40^3, 2,338 interface cells: 215
-// us a launch; 65 now with the dealt cuts, k_geometry).
-__device__ __forceinline__ double cubic_root_bracketed(double b, double c, double d, double lo, double hi) {
-  const float bf = (float)b, cf = (float)c, df = (float)d;
-  const float lf = (float)lo, hf = (float)hi;
-  float s = 0.5f * (lf + hf);
+// The smallest root t of t^3 - K t + C = 0 in double, where 0 <= C and
+// t^2 <= K / 6 (both cubic branches of a cut, see plic_a3).  With t = s C / K
+// and e = C^2 / K^3 (at most 0.12) it is e s^3 - s + 1 = 0 with s in
+// [1, 1.2], whose slope lies in [-1, -0.5]: nothing cancels, and a fixed
+// number of Newton steps is enough, three in single precision and two with
+// the value in double and the slope of the last of those (each leaves 1e-7 of
+// the error).  The cubic in the plane constant itself loses the digits of its
+// slope where the smallest normal components are small, as on a level free
+// surface: a closed form there (FP64 square root, acos and three cosines) was
+// off by up to 4e-9 at m1 ~ 1e-11, and a bracketed Newton iteration by 6e-9
+// (1e-9 near the ends of a bracket of general normals); this is off by 4e-16
+// everywhere, against quadruple precision on the host.  20 steps of a 40^3
+// FP64 run with one bubble (2,338 interface cells), whose geometry is bound
+// by the FP64 pipe: 3.06 ms with the bracketed iteration, 2.82 with this.
+__device__ __forceinline__ double cut_cubic(double K, double C) {
+  const double rk = 1.0 / K, t0 = C * rk, e = t0 * t0 * rk;
+  const float ef = (float)e;
+  float s = 1.f + ef;
 #pragma unroll
-  for (int it = 0; it < 4; ++it) {
-    const float v = ((s + bf) * s + cf) * s + df, g = (3.f * s + 2.f * bf) * s + cf;
-    s = fminf(fmaxf(s - v / g, lf), hf);
-  }
-  double a = s >= lf && s <= hf ? (double)s : 0.5 * (lo + hi);
-  a = a < lo ? lo : (a > hi ? hi : a);
-  for (int it = 0; it < 100; ++it) {
-    const double v = ((a + b) * a + c) * a + d;
-    if (v > 0.0) lo = a; else hi = a;
-    const float af = (float)a;
-    double an = a - (double)((float)v / ((3.f * af + 2.f * bf) * af + cf));
-    if (!(an >= lo && an <= hi)) an = 0.5 * (lo + hi);
-    const double step = fabs(an - a);
-    a = an;
-    // what is left is 1e-7 of the step and its square: below the roundoff
-    // of the value (which a bound near it would chase)
-    if (step <= 1e-9) break;
-  }
-  return a;
+  for (int it = 0; it < 3; ++it) s -= __fdividef((ef * s * s - 1.f) * s + 1.f, 3.f * ef * s * s - 1.f);
+  const float g = __fdividef(1.f, 3.f * ef * s * s - 1.f);
+  double x = (double)s;
+#pragma unroll
+  for (int it = 0; it < 2; ++it) x -= (double)((float)((e * x * x - 1.0) * x + 1.0) * g);
+  return t0 * x;
 }
 
 // plane constant a in [0, 1/2] of the normalised problem: gas fraction V
@@ -140,32 +130,33 @@ __device__ __forceinline__ R plic_a3(R m1, R m2, R m3, R V) {
   const R V2 = V1 + (m2 - m1) / ((R)2 * m3);
   if (V < V1) return cbrt((R)6 * m1 * m2 * m3 * V);
   if (V < V2) return (R)0.5 * m1 + sqrt((R)72 * m2 * m3 * V - (R)3 * m1 * m1) / (R)6;
-  const R six = (R)6 * m1 * m2 * m3;
   if constexpr (sizeof(R) == 8) {
-    // one solve for the cubic branches of all lanes
-    const bool over = !(m3 < m12);  // the cut reaches the far corner's planes before m3
-    const R s2 = m1 * m1 + m2 * m2, s3 = m1 * m1 * m1 + m2 * m2 * m2;
-    const R V3 = over ? m12 / ((R)2 * m3) : (m3 * m3 * ((R)3 * m12 - m3) + m1 * m1 * (m1 - (R)3 * m3) + m2 * m2 * (m2 - (R)3 * m3)) / six;
-    const bool low = V < V3;
-    if (over && !low) return m3 * V + (R)0.5 * m12;
-    const R b = low ? (R)-3 * m12 : (R)-1.5;
-    const R c = low ? (R)3 * s2 : (R)1.5 * (s2 + m3 * m3);
-    const R d = low ? -(s3 - six * V) : (R)-0.5 * (s3 + m3 * m3 * m3 - six * V);
-    return cubic_root_bracketed(b, c, d, low ? m2 : m3, low ? (over ? m12 : m3) : (R)0.5);
-  }
-  if (m3 < m12) {
-    const R V3 = (m3 * m3 * ((R)3 * m12 - m3) + m1 * m1 * (m1 - (R)3 * m3) + m2 * m2 * (m2 - (R)3 * m3)) / six;
+    // One solve for the cubic branches of all lanes.  Beyond a = m2 and below
+    // min(m3, m12), a^3 - (a - m1)^3 - (a - m2)^3 = 6 m1 m2 m3 V reads, with
+    // a = m12 - t, t^3 - 6 m1 m2 t + 3 m1 m2 (m12 - 2 m3 V) = 0; t runs down
+    // from m1 to w3 = max(m12 - m3, 0), where the cubic's sign tells the
+    // branch.  Beyond a = m3 (where m3 < m12), with a = 1/2 - t and
+    // m1 + m2 + m3 = 1: t^3 - 3 (m1 m2 - (1/2 - m3)^2) t
+    // + 3/2 m1 m2 m3 (1 - 2 V) = 0.
+    const R k = m1 * m2, q = m12 - (R)2 * m3 * V, w3 = m3 < m12 ? m12 - m3 : (R)0, h = (R)0.5 - m3;
+    const bool low = w3 * (w3 * w3 - (R)6 * k) + (R)3 * k * q > (R)0;
+    if (!low && !(m3 < m12)) return m3 * V + (R)0.5 * m12;
+    return (low ? m12 : (R)0.5) - cut_cubic(low ? (R)6 * k : (R)3 * (k - h * h),
+                                            low ? (R)3 * k * q : (R)1.5 * k * m3 * ((R)1 - (R)2 * V));
+  } else {
+    const R six = (R)6 * m1 * m2 * m3;
+    if (m3 < m12) {
+      const R V3 = (m3 * m3 * ((R)3 * m12 - m3) + m1 * m1 * (m1 - (R)3 * m3) + m2 * m2 * (m2 - (R)3 * m3)) / six;
+      if (V < V3)
+        return cubic_root_in((R)-3 * m12, (R)3 * (m1 * m1 + m2 * m2), -(m1 * m1 * m1 + m2 * m2 * m2 - six * V), m2, m3);
+      const R S2 = m1 * m1 + m2 * m2 + m3 * m3, S3 = m1 * m1 * m1 + m2 * m2 * m2 + m3 * m3 * m3;
+      return cubic_root_in((R)-1.5, (R)1.5 * S2, -(S3 - six * V) / (R)2, m3, (R)0.5);
+    }
+    const R V3 = m12 / ((R)2 * m3);
     if (V < V3)
-      return cubic_root_in<R>((R)-3 * m12, (R)3 * (m1 * m1 + m2 * m2),
-                              -(m1 * m1 * m1 + m2 * m2 * m2 - six * V), m2, m3);
-    const R S2 = m1 * m1 + m2 * m2 + m3 * m3, S3 = m1 * m1 * m1 + m2 * m2 * m2 + m3 * m3 * m3;
-    return cubic_root_in<R>((R)-1.5, (R)1.5 * S2, -(S3 - six * V) / (R)2, m3, (R)0.5);
+      return cubic_root_in((R)-3 * m12, (R)3 * (m1 * m1 + m2 * m2), -(m1 * m1 * m1 + m2 * m2 * m2 - six * V), m2, m12);
+    return m3 * V + (R)0.5 * m12;
   }
-  const R V3 = m12 / ((R)2 * m3);
-  if (V < V3)
-    return cubic_root_in<R>((R)-3 * m12, (R)3 * (m1 * m1 + m2 * m2),
-                            -(m1 * m1 * m1 + m2 * m2 * m2 - six * V), m2, m12);
-  return m3 * V + (R)0.5 * m12;
 }
 
 // PLIC inversion for one normal: the normalised, sorted components are
@@ -202,11 +193,6 @@ template <int D, class R> struct Plic {
     return a * sum - (R)0.5 * sum;
   }
 };
-
-template <int D, class R>
-__device__ __forceinline__ R plic_offset(R nx, R ny, R nz, R alpha) {
-  return Plic<D, R>(nx, ny, nz).offset(alpha);
-}
 
 // Cholesky solve of the k x k symmetric positive definite system A x = b
 // (the ridge keeps the least-squares normal matrix definite); the
