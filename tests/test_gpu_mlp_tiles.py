@@ -75,3 +75,51 @@ def test_generated_fill_levels_match_sampling(env, n):
     L.mlp_stencils_from_params(P, x, y)
     got = np.sort(x.cpu().numpy(), axis=1)
     assert np.array_equal(got, np.array(want).astype(np.float32))
+
+
+def gradient_with_roundings(th, x, t):
+    """Loss and gradient in FP64 with the operands of every product rounded
+    to BF16 as the kernel rounds them."""
+    r = mlp.bf16
+    W1, b1, W2, b2, W3, b3 = mlp.split(th)
+    n = len(x)
+    X, V1, V2 = r(x), r(W1), r(W2)
+    z1 = X @ V1.T + b1
+    H1 = r(mlp.silu(z1))
+    z2 = H1 @ V2.T + b2
+    H2 = r(mlp.silu(z2))
+    e = H2 @ W3 + b3[0] - t
+    d3 = e / n
+    d2 = r(d3[:, None] * W3 * mlp.dsilu(z2))
+    d1 = r((d2 @ V2) * mlp.dsilu(z1))
+    parts = [d1.T @ X, d1.sum(0), d2.T @ H1, d2.sum(0), H2.T @ d3, [d3.sum()]]
+    return 0.5 * np.mean(e * e), np.concatenate([np.ravel(p) for p in parts])
+
+
+@pytest.mark.parametrize("n", [1, 63, 65, 127, 128, 129, -5])
+def test_gradient_tiles(env, n):
+    """The gradient where the 128-row tiles end, and (n = -5) over two tiles
+    and a partial third of every CTA.  What is left against the same BF16
+    roundings in FP64 is FP32 sums (1e-5 of a block) and operands that round
+    the other way, 2^-8 of one in a few hundred: 2e-3 of a block's norm."""
+    L, torch = env
+    if n < 0:
+        n = 2 * 128 * torch.cuda.get_device_properties(0).multi_processor_count - n
+    rng = np.random.default_rng(n)
+    th = (mlp.init_params(6) + 0.05 * rng.normal(size=mlp.NPARAM)).astype(np.float32).astype(np.float64)
+    x = rng.random((n, 27)).astype(np.float32).astype(np.float64)
+    # residuals away from zero, more of one sign: no block cancels
+    t = (mlp.forward(th, x) + rng.uniform(1, 2, n) * np.where(rng.random(n) < 0.8, 1, -1)).astype(np.float32).astype(np.float64)
+    dev = lambda a: torch.tensor(a, dtype=torch.float32, device="cuda")  # noqa: E731
+    grad = torch.full((mlp.NPARAM + 1,), 3.0, device="cuda")
+    loss = torch.full((1,), 3.0, dtype=torch.float64, device="cuda")
+    L.mlp_loss_grad(dev(th), dev(x), dev(t), grad[:-1], loss)
+    g = grad.cpu().numpy().astype(np.float64)
+    assert g[-1] == 3.0
+    want_loss, want = gradient_with_roundings(th, x, t)
+    assert abs(loss.item() - want_loss) < 2e-3 * want_loss
+    k = 0
+    for s in mlp.SIZES:
+        m = int(np.prod(s))
+        assert np.linalg.norm(g[k:k + m] - want[k:k + m]) < 2e-3 * np.linalg.norm(want[k:k + m]), s
+        k += m
