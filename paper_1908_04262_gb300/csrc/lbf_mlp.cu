@@ -3,6 +3,7 @@
 // and backward passes, Adam, and the host entry points of include/lbf.h.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <vector>
@@ -435,10 +436,12 @@ __device__ __forceinline__ double urand(unsigned long long seed, long long i, in
   return (double)(h >> 11) * (1.0 / 9007199254740992.0);
 }
 
-__global__ void k_gen_params(unsigned long long seed, int n, double rmin, double rmax, double *par) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  double *P = par + (size_t)i * 20;
+// shapes first .. first + n of a generation
+__global__ void k_gen_params(unsigned long long seed, int first, int n, double rmin, double rmax, double *par) {
+  const int j = blockIdx.x * blockDim.x + threadIdx.x;
+  if (j >= n) return;
+  const int i = first + j;
+  double *P = par + (size_t)j * 20;
   const double R = exp(log(rmin) + urand(seed, i, 0) * (log(rmax) - log(rmin)));
   const bool ellipsoid = urand(seed, i, 1) < 0.5;
   for (int d = 0; d < 3; ++d) P[3 + d] = R * (ellipsoid ? 0.75 + 0.5 * urand(seed, i, 2 + d) : 1.0);
@@ -637,16 +640,34 @@ unsigned long long host_gcd(unsigned long long a, unsigned long long b) {
   return a;
 }
 
-// scratch of a generation: 20 doubles and a quadric per sample
-size_t gen_bytes(int n) { return (sizeof(double) * 20 + sizeof(Quadric)) * (size_t)n; }
-void gen_launch(double *par, int n, float *x, float *y, cudaStream_t st) {
-  Quadric *quad = reinterpret_cast<Quadric *>(par + (size_t)20 * n);
-  const unsigned b = (unsigned)((n + 127) / 128);
-  // one warp per sample, four a block; more than fill the GPU walk
-  const unsigned fb = (unsigned)((n + 3) / 4);
-  k_gen_quadrics<<<b, 128, 0, st>>>(par, n, quad);
-  k_gen_fill<<<fb < 1u << 15 ? fb : 1u << 15, 128, 0, st>>>(par, quad, n, x);
-  k_gen_finish<<<b, 128, 0, st>>>(par, n, x, y);
+// Generation in chunks of up to GEN_CHUNK samples, each through the same
+// scratch (20 doubles and a quadric, 280 bytes, per sample of a chunk): a run
+// over hundreds of millions of samples needs no more device memory than its
+// outputs and 294 MB.  A chunk is about 6 ms of work, so that the launches
+// between chunks do not show.
+constexpr int GEN_CHUNK = 1 << 20;
+size_t gen_bytes(int n) { return (sizeof(double) * 20 + sizeof(Quadric)) * (size_t)std::min(n, GEN_CHUNK); }
+template <class Fill> int gen_chunks(int n, float *x, float *y, cudaStream_t st, Fill fill_params) {
+  double *par = nullptr;
+  CKM(cudaMallocAsync((void **)&par, gen_bytes(n), st));
+  Quadric *quad = reinterpret_cast<Quadric *>(par + (size_t)20 * std::min(n, GEN_CHUNK));
+  cudaError_t e = cudaSuccess;
+  for (int first = 0; first < n && e == cudaSuccess; first += std::min(n - first, GEN_CHUNK)) {
+    const int m = std::min(n - first, GEN_CHUNK);
+    float *xc = x + (size_t)first * 27;
+    e = fill_params(first, m, par);
+    if (e != cudaSuccess) break;
+    const unsigned b = (unsigned)((m + 127) / 128);
+    // one warp per sample, four a block; more than fill the GPU walk
+    const unsigned fb = (unsigned)((m + 3) / 4);
+    k_gen_quadrics<<<b, 128, 0, st>>>(par, m, quad);
+    k_gen_fill<<<fb < 1u << 15 ? fb : 1u << 15, 128, 0, st>>>(par, quad, m, xc);
+    k_gen_finish<<<b, 128, 0, st>>>(par, m, xc, y + first);
+    e = cudaGetLastError();
+  }
+  CKM(cudaFreeAsync(par, st));
+  CKM(e);
+  return 0;
 }
 
 // a cleared training image made from theta
@@ -734,24 +755,19 @@ int lbf_mlp_generate(unsigned long long seed, int n, double rmin, double rmax, f
   if (!x || !y || n < 0 || !(rmin > 0) || !(rmax >= rmin)) return fail(LBF_EINVAL, "bad arguments");
   if (n == 0) return 0;
   cudaStream_t st = (cudaStream_t)stream;
-  double *par = nullptr;
-  CKM(cudaMallocAsync((void **)&par, gen_bytes(n), st));
-  k_gen_params<<<(n + 127) / 128, 128, 0, st>>>(seed, n, rmin, rmax, par);
-  gen_launch(par, n, x, y, st);
-  CKM(cudaGetLastError());
-  CKM(cudaFreeAsync(par, st));
-  return 0;
+  return gen_chunks(n, x, y, st, [&](int first, int m, double *par) {
+    k_gen_params<<<(m + 127) / 128, 128, 0, st>>>(seed, first, m, rmin, rmax, par);
+    return cudaGetLastError();
+  });
 }
 
 int lbf_mlp_stencils_from_params(const double *params, int n, float *x, float *y, void *stream) {
   if (!params || !x || !y || n <= 0) return fail(LBF_EINVAL, "bad arguments");
   cudaStream_t st = (cudaStream_t)stream;
-  double *par = nullptr;
-  CKM(cudaMallocAsync((void **)&par, gen_bytes(n), st));
-  CKM(cudaMemcpyAsync(par, params, sizeof(double) * 20 * (size_t)n, cudaMemcpyHostToDevice, st));
-  gen_launch(par, n, x, y, st);
-  CKM(cudaGetLastError());
-  CKM(cudaFreeAsync(par, st));
+  int rc = gen_chunks(n, x, y, st, [&](int first, int m, double *par) {
+    return cudaMemcpyAsync(par, params + (size_t)20 * first, sizeof(double) * 20 * (size_t)m, cudaMemcpyHostToDevice, st);
+  });
+  if (rc) return rc;
   CKM(cudaStreamSynchronize(st));
   return 0;
 }
