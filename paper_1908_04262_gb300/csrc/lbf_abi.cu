@@ -1062,6 +1062,8 @@ int lbf_create(const lbf_config *cfg, lbf_sim **out) {
   e = e ? e : cudaMemsetAsync(s->rmv, 0xff, sizeof(int), s->st);
   e = e ? e : cudaMemsetAsync(s->rmv + 1, 0, sizeof(int), s->st);
   e = e ? e : zero(s->tdirty, s->ntiles_alloc);
+  // read at roots only; no label at all where there has been none
+  e = e ? e : cudaMemsetAsync(s->rlabel, 0xff, sizeof(int) * N, s->st);
   if (e != cudaSuccess) {
     lbf_destroy(s);
     return fail(LBF_ECUDA, std::string("cudaMemsetAsync: ") + cudaGetErrorString(e));

@@ -35,6 +35,21 @@ __device__ __forceinline__ int uf_find(int *par, int a) {
   return a;
 }
 
+// The root without writes, for the pass that stores final parents
+// (k_uf_compress): there a halving write of one block, made from a parent it
+// read before, could land after the block that owns the cell had stored the
+// root, and leave that cell one link short of it.  The cell's label was then
+// whatever rlabel held at a cell that is no root, and as such cells are the
+// roots of their tiles, the tile's gas was counted to it.
+__device__ __forceinline__ int uf_root(const int *par, int a) {
+  for (int it = 0; it < UF_ITERS; ++it) {
+    const int b = __ldcg(par + a);
+    if (b == a) break;
+    a = b;
+  }
+  return a;
+}
+
 // the same on arrays that may live in shared or global memory
 __device__ __forceinline__ int uf_find_any(const int *par, int a) {
   for (int it = 0; it < UF_ITERS; ++it) {
@@ -404,7 +419,7 @@ __global__ void __launch_bounds__(TILE_THREADS) k_uf_compress(Params p) {
       const int r0 = p.troot[tile];
       __syncthreads();  // sroot of the last tile is no longer read
       if (threadIdx.x == 0) {
-        sroot = uf_find(p.parent, r0);
+        sroot = uf_root(p.parent, r0);
         if (sroot == r0) {
           const int k = atomicAdd(p.nroots, 1);
           if (k < p.cap) {
@@ -431,7 +446,7 @@ __global__ void __launch_bounds__(TILE_THREADS) k_uf_compress(Params p) {
       if (x >= p.nx || y >= p.ny || z >= p.nz) continue;
       const long long n = x + nx * y + nxy * z;
       if (post_type(p.flags[n]) != T_GAS) continue;
-      const int r = uf_find(p.parent, (int)n);
+      const int r = uf_root(p.parent, (int)n);
       p.parent[n] = r;
       if (r == (int)n) {
         const int k = atomicAdd(p.nroots, 1);
