@@ -311,89 +311,100 @@ __device__ __forceinline__ bool seg_cell_walled(const Params &p, int seg, int la
   return x < nx;
 }
 
-// A warp's share of the interface cells of the segment list, packed into
-// full warps: `batch` segments at a time, their interface cells (those whose
-// flag byte passes `take`) numbered through, 32 of them per call of `body`
-// with one cell per lane (`on` false past the last).  Foams hold 5-12
-// interface cells per segment, so one segment per warp left two thirds of
-// the lanes idle.  The batch is as large as keeps every warp of the grid
-// busy: short lists (a 128^3 foam) stay at one segment per warp, where the
-// sweep is a latency chain and packing would only lengthen it; lattices with
-// fewer segments than the grid has warps never pack (PACK false: the host's
-// choice).  Measured: 512x512x384, 663,000 interface cells in 130,000
-// segments, interface sweep 664 -> 500 us, exchange 245 -> 157 us; in the
-// 256^3 foam (104,000 in 14,300) the two alone take as long as before, but
-// the step beside the liquid sweep 640 -> 565 us, on a third of the
-// instructions.
+// position of the k-th set bit of m, k from 0 (31 past the last)
+__device__ __forceinline__ int kth_set_bit(unsigned m, int k) {
+  int q = 0;
+#pragma unroll
+  for (int h = 16; h > 0; h >>= 1) {
+    const int lo = __popc(m & ((1u << h) - 1u));
+    if (k >= lo) {
+      k -= lo;
+      q += h;
+      m >>= h;
+    }
+  }
+  return q;
+}
+
+// A warp's share of the interface cells of the segment list, one cell per
+// lane and call of `body` (`on` false for lanes without one): a segment per
+// call, or, with PACKABLE and a long list, packed into full warps: `batch`
+// segments at a time, their interface cells (those whose flag byte passes
+// `take`) numbered through, 32 of them per call.  Foams hold 5-12 interface
+// cells per segment, so one segment per warp left two thirds of the lanes
+// idle.  A warp takes its whole share as one batch, of up to 32 segments.
+//
+// Packing starts where the list fills the grid's warps four thirds over: just
+// past once, batches of two idle half the warps where single segments end in
+// a short second round (128^3, 8 bubbles, 2,813 segments on 2,432 warps: the
+// interface sweep 34 us in batches of two, 31-32 in single segments, the step
+// 131 and 126).  The two loops have a body each, which keeps the short one
+// free of the other's bookkeeping (in one loop it ran at 32-33 us).
+// Measured, packed against single segments: 512x512x384, 663,000 interface
+// cells in 130,000 segments, interface sweep 664 -> 500 us, exchange 245 ->
+// 157 us; 128^3 with 180 bubbles (22,100 segments) the step 324 -> 294 us in
+// FP32 and 327 -> 284 in shifted FP16; in the 256^3 foam (104,000 in 14,300)
+// the two alone take as long either way, but the step beside the liquid
+// sweep 640 -> 565 us, on a third of the instructions.  In 2D no list was
+// long enough (450x650: at most one segment per warp): not compiled there.
 // s_mask, s_first: 32 words each of the warp's shared memory.
-template <bool WALLED, bool PACK, class Take, class Body>
+template <bool WALLED, bool PACKABLE, class Take, class Body>
 __device__ __forceinline__ void for_segment_cells(const Params &p, const int *seglist, int cnt, unsigned *s_mask,
                                                   unsigned *s_first, Take take, Body body) {
   const int lane = threadIdx.x & 31;
   const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nwarps = (gridDim.x * blockDim.x) >> 5;
-  const int batch = PACK ? min(32, max(1, (cnt + nwarps - 1) / nwarps)) : 1;
+  if (!PACKABLE || 3ll * cnt < 4ll * nwarps) {
+    for (int k = warp; k < cnt; k += nwarps) {
+      Cell c;
+      const bool inr = WALLED ? seg_cell_walled(p, seglist[k], lane, c) : seg_cell(p, seglist[k], lane, c);
+      body(c, inr && take(p.flags[c.n]));
+    }
+    return;
+  }
+  const int batch = min(32, (cnt + nwarps - 1) / nwarps);
   const int nxb = (p.nx + 31) >> 5;
   for (int base = warp * batch; base < cnt; base += nwarps * batch) {
     const int ns = min(batch, cnt - base);
     const int myseg = seglist[base + min(lane, ns - 1)];
-    unsigned total = 32;
-    if (batch > 1) {
-      unsigned mine = 0;
-      for (int s0 = 0; s0 < ns; s0 += 8) {
-        uint8_t fl[8];
+    unsigned mine = 0;
+    for (int s0 = 0; s0 < ns; s0 += 8) {
+      uint8_t fl[8];
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          const int seg = __shfl_sync(0xffffffffu, myseg, (s0 + j) & 31);
-          const int row = seg / nxb, x = (seg - row * nxb) * 32 + lane;
-          fl[j] = (s0 + j < ns && x < p.nx) ? p.flags[x + p.nx * row] : (uint8_t)T_WALL;
-        }
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          const unsigned m = __ballot_sync(0xffffffffu, take(fl[j]));
-          if (lane == s0 + j) mine = m;
-        }
+      for (int j = 0; j < 8; ++j) {
+        const int seg = __shfl_sync(0xffffffffu, myseg, (s0 + j) & 31);
+        const int row = seg / nxb, x = (seg - row * nxb) * 32 + lane;
+        fl[j] = (s0 + j < ns && x < p.nx) ? p.flags[x + p.nx * row] : (uint8_t)T_WALL;
       }
-      unsigned incl = (unsigned)__popc(mine);
-      const unsigned own = incl;
 #pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const unsigned v = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += v;
+      for (int j = 0; j < 8; ++j) {
+        const unsigned m = __ballot_sync(0xffffffffu, take(fl[j]));
+        if (lane == s0 + j) mine = m;
       }
-      total = __shfl_sync(0xffffffffu, incl, 31);
-      s_mask[lane] = mine;
-      s_first[lane] = incl - own;
-      __syncwarp();
     }
+    unsigned incl = (unsigned)__popc(mine);
+    const unsigned own = incl;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned v = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += v;
+    }
+    const unsigned total = __shfl_sync(0xffffffffu, incl, 31);
+    s_mask[lane] = mine;
+    s_first[lane] = incl - own;
+    __syncwarp();
     for (unsigned c0 = 0; c0 < total; c0 += 32) {
       const unsigned k = c0 + lane;
-      bool on = k < total;
-      int sg = 0, bit = lane;
-      if (batch > 1) {
-        // the segment that holds cell k: the last whose first cell is <= k
-        // (segments without cells share their successor's first and lose)
+      const bool on = k < total;
+      // the segment that holds cell k: the last whose first cell is <= k
+      // (segments without cells share their successor's first and lose)
+      int sg = 0;
 #pragma unroll
-        for (int h = 16; h > 0; h >>= 1)
-          if (s_first[sg + h] <= k) sg += h;
-        // its (k - first)-th set bit
-        unsigned m = s_mask[sg];
-        int j = on ? (int)(k - s_first[sg]) : 0;
-        bit = 0;
-#pragma unroll
-        for (int h = 16; h > 0; h >>= 1) {
-          const int lo = __popc(m & ((1u << h) - 1u));
-          if (j >= lo) {
-            j -= lo;
-            bit += h;
-            m >>= h;
-          }
-        }
-        if (!on) bit = 0;
-      }
+      for (int h = 16; h > 0; h >>= 1)
+        if (s_first[sg + h] <= k) sg += h;
+      const int kth = kth_set_bit(s_mask[sg], on ? (int)(k - s_first[sg]) : 0), bit = on ? kth : 0;
       const int seg = __shfl_sync(0xffffffffu, myseg, sg);
       Cell c;
-      const bool inr = WALLED ? seg_cell_walled(p, seg, bit, c) : seg_cell(p, seg, bit, c);
-      if (batch == 1) on = inr && take(p.flags[c.n]);
+      if (WALLED) seg_cell_walled(p, seg, bit, c); else seg_cell(p, seg, bit, c);
       body(c, on);
     }
     __syncwarp();

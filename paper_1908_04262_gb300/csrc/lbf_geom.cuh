@@ -347,18 +347,7 @@ __global__ void __launch_bounds__(128, sizeof(R) == 4 ? 8 : 4) k_geometry(Params
       R *sc = s_cut[threadIdx.x >> 5][sub];
       const int ncut = __popc(cuts);
       for (int k = t; __any_sync(0xffffffffu, k < ncut); k += G) {
-        // the k-th set bit
-        unsigned m = cuts;
-        int j = k, q = 0;
-#pragma unroll
-        for (int h = 16; h > 0; h >>= 1) {
-          const int lo = __popc(m & ((1u << h) - 1u));
-          if (j >= lo) {
-            j -= lo;
-            q += h;
-            m >>= h;
-          }
-        }
+        const int q = kth_set_bit(cuts, k);
         if (k < ncut) sc[q] = plic.offset(sc[q]);
       }
       __syncwarp();

@@ -51,19 +51,11 @@ struct OpsImpl final : Ops {
     k_nucleate<D, S><<<blocks_for(cnt, B), B, 0, s>>>(p, par, c[0], c[1], D == 3 ? c[2] : 0.0, R0, x0, y0,
                                                         z0, bx, by, bz);
   }
-  // more segments than the grid has warps (four a block)
-  static bool packs(const Params &p, int blocks) {
-    return (long long)((p.nx + 31) / 32) * p.ny * p.nz > 4ll * blocks;
-  }
-  template <bool WALLED, bool PACK> void exchange_as(const Params &p, int par, cudaStream_t s) {
-    par ? k_exchange<D, S, 1, WALLED, PACK><<<p.warp_blocks, 128, 0, s>>>(p)
-        : k_exchange<D, S, 0, WALLED, PACK><<<p.warp_blocks, 128, 0, s>>>(p);
-  }
   void exchange(const Params &p, int par, cudaStream_t s) override {
-    if (packs(p, p.warp_blocks))
-      p.walled ? exchange_as<true, true>(p, par, s) : exchange_as<false, true>(p, par, s);
+    if (p.walled)
+      par ? k_exchange<D, S, 1, true><<<p.warp_blocks, 128, 0, s>>>(p) : k_exchange<D, S, 0, true><<<p.warp_blocks, 128, 0, s>>>(p);
     else
-      p.walled ? exchange_as<true, false>(p, par, s) : exchange_as<false, false>(p, par, s);
+      par ? k_exchange<D, S, 1><<<p.warp_blocks, 128, 0, s>>>(p) : k_exchange<D, S, 0><<<p.warp_blocks, 128, 0, s>>>(p);
   }
   void build_ilist(const Params &p, cudaStream_t s) override {
     cudaMemsetAsync(p.icount, 0, sizeof(int), s);
@@ -87,12 +79,8 @@ struct OpsImpl final : Ops {
   }
   template <int COLL, bool WALLED> void interface_as(const Params &p, int par, cudaStream_t s) {
     const int g = p.list_blocks;
-    if (packs(p, g))
-      par ? k_stream_interface<D, S, 1, COLL, WALLED, true><<<g, 128, 0, s>>>(p)
-          : k_stream_interface<D, S, 0, COLL, WALLED, true><<<g, 128, 0, s>>>(p);
-    else
-      par ? k_stream_interface<D, S, 1, COLL, WALLED, false><<<g, 128, 0, s>>>(p)
-          : k_stream_interface<D, S, 0, COLL, WALLED, false><<<g, 128, 0, s>>>(p);
+    par ? k_stream_interface<D, S, 1, COLL, WALLED><<<g, 128, 0, s>>>(p)
+        : k_stream_interface<D, S, 0, COLL, WALLED><<<g, 128, 0, s>>>(p);
   }
   void stream_interface(const Params &p, int par, cudaStream_t s) override {
     if (p.coll == 2)
