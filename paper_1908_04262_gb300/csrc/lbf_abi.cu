@@ -317,10 +317,18 @@ void enqueue_label_sync(lbf_sim *s, const Params &p) {
 // Lattices of up to this many cells take the flag rewrite off the chain from
 // the interface sweep to the disjoining pressure: there the step is that
 // chain.  Larger ones are paced by the liquid sweep, with which an earlier
-// geometry only competes.  Measured, ms for 20 steps with and without the
-// rewrite on the chain: 2D 128^2 FP64 0.99, 0.95; 40^3 FP64 3.40, 2.91; 2D
-// 450x650 FP32 1.17, 1.20; at 128^3 4 % the other way.
+// geometry only competes; in 2D in single precision the geometry is too short
+// for its earlier start to show.  Measured, us a step with the rewrite on the
+// chain, off it:
+//            32^3        48^3        50^3       128^2       256^2       360^2
+//   FP64  151   138   290   295   335   331   51.5  48.6  67.6  64.3  78.0  78.8
+//   FP32  40.2  39.3  43.5  43.9  52.1  51.6  35.2  35.4  39.3  39.8  40.9  41.5
+//   FP16  44.4  43.4  45.2  44.6  52.1  50.8  36.1  36.2  39.9  40.8  41.9  43.0
+// and above the line, 450x650 FP32 58.5, 60.0, 128^3 4 % slower off it.
 constexpr long long kSmallLattice = 1ll << 17;
+bool early_geometry_pays(const lbf_sim *s) {
+  return s->mlp_theta != nullptr || (s->N <= kSmallLattice && (s->dim == 3 || s->cfg.storage == LBF_FP64));
+}
 
 // everything of a step after its interface sweep.  The marking runs first;
 // then every cell's post-conversion type is known and the union-find passes
@@ -354,7 +362,7 @@ void enqueue_after_sweep(lbf_sim *s, const Params &p, int par, bool waitx, const
   if (waitx) cudaStreamWaitEvent(s->st2, s->joinx, 0);
   s->ops->convert_excess(p, par, s->st2);
   cudaEventRecord(s->applied, s->st2);
-  const bool early_geometry = s->mlp_theta != nullptr || s->N <= kSmallLattice;
+  const bool early_geometry = early_geometry_pays(s);
   if (!early_geometry) {
     cudaStreamWaitEvent(s->st2, s->checked, 0);
     s->ops->convert_finalize(p, s->st2);
