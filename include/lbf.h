@@ -201,7 +201,10 @@ int lbf_ledger(lbf_sim *s, double *out8);
  * run where it was saved.
  * lbf_checkpoint_bytes: *bytes = size of the checkpoint.
  * lbf_checkpoint_save: writes it to host memory dst (bytes >= that size);
- *   synchronises.  Errors: LBF_EINVAL, LBF_ECUDA.
+ *   synchronises.  The labels and the bubble table are put in root order
+ *   first, on the device, and the next step copies every label instead of the
+ *   changed ones (both small beside the copy to the host); the run itself goes
+ *   on as without it.  Errors: LBF_EINVAL, LBF_ECUDA.
  * lbf_checkpoint_load: restores from host memory src (bytes long);
  *   synchronises.  Errors: LBF_EINVAL (not a checkpoint, too short, another
  *   lattice or storage, the learned curvature attached differently or with

@@ -124,7 +124,8 @@ struct Params {
   int *mlist, *mcount;   // interface cells the sweep marked to fill or empty this step
                          // (the count is kept per parity: see make_params)
   // 32-cell segments along x that hold interface cells (the interface
-  // kernels run one warp per segment, one lane per cell)
+  // kernels run one lane per cell: a warp per segment, or several segments'
+  // cells packed into full warps, see for_segment_cells)
   int *seglist, *segcount;       // at the start of the step
   int *segnext, *segnext_count;  // after the conversion
   int *segflag;                  // per segment: 1 while listed in segnext (the interface sweep clears it)

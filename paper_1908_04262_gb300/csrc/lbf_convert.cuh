@@ -278,7 +278,7 @@ __device__ __forceinline__ bool removal_keeps_bubble(const Params &p, const Cell
 // (64 KB of flags in 16-byte loads, labels read at gas cells only) finds it.
 // Reaching to the end of the next plane, for any number of bubbles a step
 // (the limits had been 32,768 cells and one bubble), is one of the two things
-// that keep large foams on the patched labelling: see label_fast.
+// that keep large foams on the patched labelling: see patch_labels.
 //
 // The last block to finish writes the step's choice of labelling branch,
 // lab_fast: patched unless the state was set from outside (gas_dirty -1), a
@@ -315,10 +315,20 @@ template <int D> __device__ __forceinline__ int patched_label(const Params &p, i
   return knew;
 }
 
-// Root moves that renumber: two bubbles lost their root cells, one lost it
-// while a root was lowered, a moved root passed another's, or the new root
-// lies more than 32,768 cells on.  (Fewer moves leave each bubble its gas
-// whatever an interface cell's label does.)  Whole block.
+// Root moves after which two bubbles that come to share an interface cell
+// pool their gas: two bubbles lost their root cells, one lost it while a root
+// was lowered, a moved root passed another's, or the new root lies more than
+// 32,768 cells on.  This is no rule of the model.  It repeats the cases in
+// which the labelling by root ranks, with its scan of 32,768 cells, gave up
+// and took the full labelling, so that runs keep the ids and pressures they
+// had.  By the model (Sec. 3.5 as the CPU reference reads it: old and new
+// bubbles join over every cell they share) any interface cell that changes
+// its bubble is enough; a gas neighbour that turns interface does that
+// without moving a root, and such a step is patched here and each bubble
+// keeps its gas: 32^3, bubbles of radius 5 and 3 behind one interface layer,
+// ids [1, 3] after 9 steps where the reference has [1, 4].  `fast = false`
+// for every changed cell gives the reference's results at no measured cost.
+// Whole block.
 __device__ __forceinline__ bool renumbers(const Params &p, int removed) {
   if (removed >= 2 || (removed == 1 && p.rmv[1])) return true;
   const int cnt = *p.told.count;

@@ -742,10 +742,13 @@ static __global__ void __launch_bounds__(1024) k_bubble_update(Params p) {
 // added gas cells (the label they had as interface cells, which is their
 // bubble's) and the interface cells after the conversion (the gas neighbour
 // whose bubble has the smallest root).  Root cells move as bubbles grow and
-// deform; the labels do not change with them.  The result equals the full
-// labelling's once slots are read through their ranks.  The step graph picks
-// this branch or the full one on the device (k_root_scan writes lab_fast):
-// the union-find kernels return at once, the others take the branch inside.
+// deform; the labels do not change with them.  Flags, labels and the shape of
+// the bubble table equal the full labelling's once slots are read through
+// their ranks; so do ids and gas, except that bubbles which come to share an
+// interface cell pool their gas only where `renumbers` sends the step to the
+// full labelling.  The step graph picks this branch or the full one on the
+// device (k_root_scan writes lab_fast): the union-find kernels return at once,
+// the others take the branch inside.
 //
 // Why slots: with the labels themselves in root order, every root that moved
 // past another's, and every second root moved in a step, forced a full

@@ -40,13 +40,13 @@ int fail(int code, const char *msg) {
 // special-function unit, two results for each of the 128 SiLUs of a row
 // (27 us at 503,117 rows).  Measured there: 208 -> 68 us, and 50 with the
 // inputs staged as below.
-constexpr int FWD_THREADS = 256, FWD_CTAS = 4;
 //
 // The inputs of a full tile are 13,824 consecutive bytes: one bulk copy
 // brings them into shared memory while the tile before is worked on, and
 // each thread packs half a row from there (27 words apart, no bank
 // conflicts) into two 16-byte pieces of the operand.  The last, partial tile
 // and inputs that do not start on 16 bytes are gathered with plain loads.
+constexpr int FWD_THREADS = 256, FWD_CTAS = 4;
 struct __align__(128) FwdSmem {
   tc::Tile t;
   float x[tc::ROWS * 27];
@@ -708,7 +708,6 @@ size_t image_bytes() { return sizeof(tc::Image); }
 void pack_launch(const float *theta, void *img, cudaStream_t st) {
   k_pack_net<<<1, 256, 0, st>>>(theta, (tc::Image *)img);
 }
-// in-loop use by the simulation (declared in lbf_ops_api.h)
 void forward_launch(const float *theta, const float *x, int n, float *y, cudaStream_t st) {
   const int tiles = (n + tc::ROWS - 1) / tc::ROWS;
   int dev = 0, sms = 0;

@@ -121,7 +121,9 @@ struct OpsImpl final : Ops {
   }
   void label_relabel(const Params &p, cudaStream_t s) override {
     // four blocks per SM for the patch's short lists; the full relabelling
-    // walks every segment of the lattice with them
+    // walks every segment of the lattice with them (carving a nucleus, which
+    // labels in full: 256^3 1.00 ms a call, 128^3 0.30; with 16 blocks per SM
+    // 1.01 and 0.30)
     k_relabel<D, R><<<p.list_blocks, 128, 0, s>>>(p);
   }
   void bubble_update(const Params &p, cudaStream_t s) override { k_bubble_update<<<1, 1024, 0, s>>>(p); }
