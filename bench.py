@@ -123,7 +123,7 @@ def stop_clocks(proc, path):
 # were profiled
 SWEEP_TRAFFIC_BYTES = 264.1e6
 SWEEP_SOURCES = ("paper_1908_04262_gb300/csrc/lbf_stream.cuh", "paper_1908_04262_gb300/csrc/lbf_common.cuh")
-SWEEP_SOURCES_SHA256_16 = "92892d233b1f8963"
+SWEEP_SOURCES_SHA256_16 = "7ac1ef4992f2c4f2"
 
 
 def sweep_traffic():

@@ -329,33 +329,47 @@ __device__ __forceinline__ int kth_set_bit(unsigned m, int k) {
 
 // A warp's share of the interface cells of the segment list, one cell per
 // lane and call of `body` (`on` false for lanes without one): a segment per
-// call, or, with PACKABLE and a long list, packed into full warps: `batch`
-// segments at a time, their interface cells (those whose flag byte passes
-// `take`) numbered through, 32 of them per call.  Foams hold 5-12 interface
-// cells per segment, so one segment per warp left two thirds of the lanes
-// idle.  A warp takes its whole share as one batch, of up to 32 segments.
+// call, or, where the list is long, packed into full warps: `batch` segments
+// at a time, their interface cells (those whose flag byte passes `take`)
+// numbered through, 32 of them per call.  Foams hold 5-12 interface cells per
+// segment, so one segment per warp left two thirds of the lanes idle.  A warp
+// takes its whole share as one batch, of up to 32 segments.
 //
-// Packing starts where the list fills the grid's warps four thirds over: just
-// past once, batches of two idle half the warps where single segments end in
-// a short second round (128^3, 8 bubbles, 2,813 segments on 2,432 warps: the
-// interface sweep 34 us in batches of two, 31-32 in single segments, the step
-// 131 and 126).  The two loops have a body each, which keeps the short one
-// free of the other's bookkeeping (as one loop the step took 128 us, and 109.6
-// for 108.8 in shifted FP16).
-// Measured, packed against single segments: 512x512x384, 663,000 interface
-// cells in 130,000 segments, interface sweep 664 -> 500 us, exchange 245 ->
-// 157 us; 128^3 with 180 bubbles (22,100 segments) the step 324 -> 294 us in
-// FP32 and 327 -> 284 in shifted FP16; in the 256^3 foam (104,000 in 14,300)
-// the two alone take as long either way, but the step beside the liquid
-// sweep 640 -> 565 us, on a third of the instructions.  In 2D no list was
-// long enough (450x650: at most one segment per warp): not compiled there.
+// Packing starts with a list longer than the grid's warps (EARLY), in the
+// single-precision and 16-bit interface sweeps where it fills them four thirds
+// over: their body is a long chain of latencies, and just past once batches of
+// two idle half the warps where single segments end in a short second round
+// (128^3, 8 bubbles, 2,813 segments on 2,432 warps: the sweep 34 us in batches
+// of two, 32 in single segments, the step 131 and 126).  The exchange and the
+// FP64 sweep, short or bound by the FP64 pipe, gain from full lanes at once
+// (2D 2000x1500, 11,800 segments on the exchange's 9,728 warps: the FP64 step
+// 764 us, 783 from four thirds on).  Measured, packed against single segments:
+// 512x512x384, 663,000 interface cells in 130,000 segments, interface sweep
+// 664 -> 500 us, exchange 245 -> 157 us; 128^3 with 180 bubbles (22,100
+// segments) the step 324 -> 294 us; 2000x1500 in FP64 909 -> 764; in the 256^3
+// foam (104,000 cells in 14,300 segments) the two alone take as long either
+// way, but the step beside the liquid sweep 640 -> 565 us, on a third of the
+// instructions.
+//
+// SEGS_TWO walks short and long lists in a loop (and a copy of the body) each,
+// SEGS_ONE in one, which leaves the short one the other's bookkeeping but has
+// the registers for one body.  Steps in one loop, two: 128^3 FP32 128, 126 us,
+// with 180 bubbles 300, 294; shifted FP16 112.6, 112.0, with the network 136.4,
+// 133.9, with 180 bubbles 246.5, 250; FP64 the same.  So the 16-bit forms take
+// one loop, the others two, and the 16-bit forms none (SEGS_SINGLE) on lattices
+// too small for a list that packs.
 // s_mask, s_first: 32 words each of the warp's shared memory.
-template <bool WALLED, bool PACKABLE, class Take, class Body>
+enum { SEGS_SINGLE = 0, SEGS_ONE = 1, SEGS_TWO = 2 };
+template <bool EARLY> __host__ __device__ constexpr bool segs_pack(long long segments, long long warps) {
+  return EARLY ? segments > warps : 3 * segments >= 4 * warps;
+}
+template <bool EARLY, bool WALLED, int SEGS, class Take, class Body>
 __device__ __forceinline__ void for_segment_cells(const Params &p, const int *seglist, int cnt, unsigned *s_mask,
                                                   unsigned *s_first, Take take, Body body) {
   const int lane = threadIdx.x & 31;
   const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nwarps = (gridDim.x * blockDim.x) >> 5;
-  if (!PACKABLE || 3ll * cnt < 4ll * nwarps) {
+  const bool pack = segs_pack<EARLY>(cnt, nwarps);
+  if (SEGS == SEGS_SINGLE || (SEGS == SEGS_TWO && !pack)) {
     for (int k = warp; k < cnt; k += nwarps) {
       Cell c;
       const bool inr = WALLED ? seg_cell_walled(p, seglist[k], lane, c) : seg_cell(p, seglist[k], lane, c);
@@ -363,50 +377,58 @@ __device__ __forceinline__ void for_segment_cells(const Params &p, const int *se
     }
     return;
   }
-  const int batch = min(32, (cnt + nwarps - 1) / nwarps);
+  const int batch = pack ? min(32, (cnt + nwarps - 1) / nwarps) : 1;
+  const bool packed = SEGS == SEGS_TWO || batch > 1;
   const int nxb = (p.nx + 31) >> 5;
   for (int base = warp * batch; base < cnt; base += nwarps * batch) {
     const int ns = min(batch, cnt - base);
     const int myseg = seglist[base + min(lane, ns - 1)];
-    unsigned mine = 0;
-    for (int s0 = 0; s0 < ns; s0 += 8) {
-      uint8_t fl[8];
+    unsigned total = 32;
+    if (packed) {
+      unsigned mine = 0;
+      for (int s0 = 0; s0 < ns; s0 += 8) {
+        uint8_t fl[8];
 #pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        const int seg = __shfl_sync(0xffffffffu, myseg, (s0 + j) & 31);
-        const int row = seg / nxb, x = (seg - row * nxb) * 32 + lane;
-        fl[j] = (s0 + j < ns && x < p.nx) ? p.flags[x + p.nx * row] : (uint8_t)T_WALL;
+        for (int j = 0; j < 8; ++j) {
+          const int seg = __shfl_sync(0xffffffffu, myseg, (s0 + j) & 31);
+          const int row = seg / nxb, x = (seg - row * nxb) * 32 + lane;
+          fl[j] = (s0 + j < ns && x < p.nx) ? p.flags[x + p.nx * row] : (uint8_t)T_WALL;
+        }
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          const unsigned m = __ballot_sync(0xffffffffu, take(fl[j]));
+          if (lane == s0 + j) mine = m;
+        }
       }
+      unsigned incl = (unsigned)__popc(mine);
+      const unsigned own = incl;
 #pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        const unsigned m = __ballot_sync(0xffffffffu, take(fl[j]));
-        if (lane == s0 + j) mine = m;
+      for (int o = 1; o < 32; o <<= 1) {
+        const unsigned v = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += v;
       }
+      total = __shfl_sync(0xffffffffu, incl, 31);
+      s_mask[lane] = mine;
+      s_first[lane] = incl - own;
+      __syncwarp();
     }
-    unsigned incl = (unsigned)__popc(mine);
-    const unsigned own = incl;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const unsigned v = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += v;
-    }
-    const unsigned total = __shfl_sync(0xffffffffu, incl, 31);
-    s_mask[lane] = mine;
-    s_first[lane] = incl - own;
-    __syncwarp();
     for (unsigned c0 = 0; c0 < total; c0 += 32) {
       const unsigned k = c0 + lane;
-      const bool on = k < total;
-      // the segment that holds cell k: the last whose first cell is <= k
-      // (segments without cells share their successor's first and lose)
-      int sg = 0;
+      bool on = k < total;
+      int sg = 0, bit = lane;
+      if (packed) {
+        // the segment that holds cell k: the last whose first cell is <= k
+        // (segments without cells share their successor's first and lose)
 #pragma unroll
-      for (int h = 16; h > 0; h >>= 1)
-        if (s_first[sg + h] <= k) sg += h;
-      const int kth = kth_set_bit(s_mask[sg], on ? (int)(k - s_first[sg]) : 0), bit = on ? kth : 0;
+        for (int h = 16; h > 0; h >>= 1)
+          if (s_first[sg + h] <= k) sg += h;
+        bit = kth_set_bit(s_mask[sg], on ? (int)(k - s_first[sg]) : 0);
+        if (!on) bit = 0;
+      }
       const int seg = __shfl_sync(0xffffffffu, myseg, sg);
       Cell c;
-      if (WALLED) seg_cell_walled(p, seg, bit, c); else seg_cell(p, seg, bit, c);
+      const bool inr = WALLED ? seg_cell_walled(p, seg, bit, c) : seg_cell(p, seg, bit, c);
+      if (!packed) on = inr && take(p.flags[c.n]);
       body(c, on);
     }
     __syncwarp();

@@ -51,11 +51,25 @@ struct OpsImpl final : Ops {
     k_nucleate<D, S><<<blocks_for(cnt, B), B, 0, s>>>(p, par, c[0], c[1], D == 3 ? c[2] : 0.0, R0, x0, y0,
                                                         z0, bx, by, bz);
   }
-  void exchange(const Params &p, int par, cudaStream_t s) override {
-    if (p.walled)
-      par ? k_exchange<D, S, 1, true><<<p.warp_blocks, 128, 0, s>>>(p) : k_exchange<D, S, 0, true><<<p.warp_blocks, 128, 0, s>>>(p);
+  // whether a grid of so many blocks (four warps each) could meet a list long
+  // enough to be packed (see for_segment_cells)
+  template <bool EARLY> static bool packs(const Params &p, int blocks) {
+    return segs_pack<EARLY>((long long)((p.nx + 31) / 32) * p.ny * p.nz, 4ll * blocks);
+  }
+  template <bool WALLED, int SEGS> void exchange_as(const Params &p, int par, cudaStream_t s) {
+    par ? k_exchange<D, S, 1, WALLED, SEGS><<<p.warp_blocks, 128, 0, s>>>(p)
+        : k_exchange<D, S, 0, WALLED, SEGS><<<p.warp_blocks, 128, 0, s>>>(p);
+  }
+  template <bool WALLED> void exchange_walled(const Params &p, int par, cudaStream_t s) {
+    if constexpr (sizeof(S) >= 4)
+      exchange_as<WALLED, SEGS_TWO>(p, par, s);
+    else if (packs<true>(p, p.warp_blocks))
+      exchange_as<WALLED, SEGS_ONE>(p, par, s);
     else
-      par ? k_exchange<D, S, 1><<<p.warp_blocks, 128, 0, s>>>(p) : k_exchange<D, S, 0><<<p.warp_blocks, 128, 0, s>>>(p);
+      exchange_as<WALLED, SEGS_SINGLE>(p, par, s);
+  }
+  void exchange(const Params &p, int par, cudaStream_t s) override {
+    p.walled ? exchange_walled<true>(p, par, s) : exchange_walled<false>(p, par, s);
   }
   void build_ilist(const Params &p, cudaStream_t s) override {
     cudaMemsetAsync(p.icount, 0, sizeof(int), s);
@@ -77,10 +91,17 @@ struct OpsImpl final : Ops {
     else
       par ? k_stream_liquid<D, S, 1, 0><<<g, b, 0, s>>>(p) : k_stream_liquid<D, S, 0, 0><<<g, b, 0, s>>>(p);
   }
+  template <int COLL, bool WALLED, int SEGS> void interface_segs(const Params &p, int par, cudaStream_t s) {
+    par ? k_stream_interface<D, S, 1, COLL, WALLED, SEGS><<<p.list_blocks, 128, 0, s>>>(p)
+        : k_stream_interface<D, S, 0, COLL, WALLED, SEGS><<<p.list_blocks, 128, 0, s>>>(p);
+  }
   template <int COLL, bool WALLED> void interface_as(const Params &p, int par, cudaStream_t s) {
-    const int g = p.list_blocks;
-    par ? k_stream_interface<D, S, 1, COLL, WALLED><<<g, 128, 0, s>>>(p)
-        : k_stream_interface<D, S, 0, COLL, WALLED><<<g, 128, 0, s>>>(p);
+    if constexpr (sizeof(S) >= 4)
+      interface_segs<COLL, WALLED, SEGS_TWO>(p, par, s);
+    else if (packs<sizeof(S) == 8>(p, p.list_blocks))
+      interface_segs<COLL, WALLED, SEGS_ONE>(p, par, s);
+    else
+      interface_segs<COLL, WALLED, SEGS_SINGLE>(p, par, s);
   }
   void stream_interface(const Params &p, int par, cudaStream_t s) override {
     if (p.coll == 2)

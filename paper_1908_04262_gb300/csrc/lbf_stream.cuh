@@ -114,7 +114,7 @@ template <class R> __device__ __forceinline__ R solve_tau(const Params &p, R A) 
 
 // the cells of the segment list, one lane each (neighbours along x coalesce
 // like the lattice sweep's)
-template <int D, class S, int PAR, bool WALLED = false>
+template <int D, class S, int PAR, bool WALLED, int SEGS>
 __global__ void __launch_bounds__(128) k_exchange(Params p) {
   using R = typename ST<S>::R;
   constexpr int Q = Lat<D>::Q;
@@ -129,7 +129,7 @@ __global__ void __launch_bounds__(128) k_exchange(Params p) {
   // types through the last conversion's marks: the exchange may run while
   // that conversion still writes the new types
   auto take = [](uint8_t fl) { return post_type(fl) == T_IFC; };
-  for_segment_cells<WALLED, D == 3>(p, p.seglist, cnt, s_mask + wb, s_first + wb, take, [&](const Cell &c, bool on) {
+  for_segment_cells<true, WALLED, SEGS>(p, p.seglist, cnt, s_mask + wb, s_first + wb, take, [&](const Cell &c, bool on) {
     if (!on) return;
     const int n = c.n;
     const R phn = phi[n];
@@ -657,7 +657,7 @@ __device__ __forceinline__ int interface_cell(const Params &p, const Cell &c, lo
 // the interface cells of the step, one lane each (for_segment_cells); cells
 // that fill or empty are listed for the conversion.  Block 0 also resets the
 // counters of the lists that the conversion fills.
-template <int D, class S, int PAR, int COLL, bool WALLED = false>
+template <int D, class S, int PAR, int COLL, bool WALLED, int SEGS>
 __global__ void __launch_bounds__(128, 4) k_stream_interface(Params p) {
   __shared__ double wbuf[128];
   __shared__ unsigned s_mask[128], s_first[128];
@@ -671,7 +671,7 @@ __global__ void __launch_bounds__(128, 4) k_stream_interface(Params p) {
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < cnt; k += gridDim.x * blockDim.x) p.segflag[p.seglist[k]] = 0;
   const int wb = threadIdx.x & ~31;
   auto take = [](uint8_t fl) { return ftype(fl) == T_IFC; };
-  for_segment_cells<WALLED, D == 3>(p, p.seglist, cnt, s_mask + wb, s_first + wb, take, [&](const Cell &c, bool on) {
+  for_segment_cells<sizeof(S) == 8, WALLED, SEGS>(p, p.seglist, cnt, s_mask + wb, s_first + wb, take, [&](const Cell &c, bool on) {
     double flux = 0.0;
     int lab = -1, mk = MK_NONE;
     if (on) mk = interface_cell<D, S, PAR, COLL>(p, c, c.n, p.flags[c.n], flux, lab);
